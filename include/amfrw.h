@@ -213,8 +213,10 @@ int amfrw_batch_run(amfrw_batch *b, double *d_prices_out);
 int amfrw_batch_launches(const amfrw_batch *b, int32_t *n_launches);
 
 /* Kernel timing (tracing).  With timing on, every amfrw_batch_run records a
- * CUDA event pair around each solver launch: one persistent multi-class
- * launch per (N, precision) for all grids of at most 64 Inner nodes (when
+ * CUDA event pair around each solver launch: one launch per (N, precision) for
+ * the grids of at most 64 Inner nodes that are solved as bundles (large
+ * batches: up to 32 instances of one grid together), one persistent
+ * multi-class launch per (N, precision) for the other grids of that size (when
  * that strategy is selected), and one launch per remaining (N, precision,
  * grid class).  amfrw_batch_kernel_times synchronises and writes, for the
  * last run, the device milliseconds of each solver launch to

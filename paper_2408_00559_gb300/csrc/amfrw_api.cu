@@ -240,6 +240,12 @@ LaunchFn launch_for(int N)
                                  launch_n5, launch_n6, launch_n7, launch_n8};
     return t[N];
 }
+BundleFn launch_bundle_for(int N)
+{
+    static const BundleFn t[] = {nullptr, nullptr, launch_bundle_n2, launch_bundle_n3, launch_bundle_n4,
+                                 launch_bundle_n5, launch_bundle_n6, launch_bundle_n7, launch_bundle_n8};
+    return t[N];
+}
 OccFn occ_for(int N)
 {
     static const OccFn t[] = {nullptr, nullptr, occupancy_n2, occupancy_n3, occupancy_n4,
@@ -275,7 +281,28 @@ struct LaunchClass {
     int64_t lu_stride;   // bytes of scratch per block: Thomas factors (CTA
                          // groups) or the whole grid state (global-memory groups)
     int64_t lu_offset;   // this class's part of the plan's scratch array
+    // warp-group classes: the grids solved as bundles come first, the warp
+    // groups take the rest (rest_begin, rest_count)
+    int bundle_begin, bundle_count;
+    int rest_begin, rest_count;
+    int bundle_smem;     // dynamic shared bytes per warp of the class's bundles
+    int bundle_lu;       // bytes of global scratch per bundle (line-solve factors that do not fit)
 };
+
+// Grids of one shape that are solved as bundles, one instance per lane: full
+// bundles of 32, and a last one of at least this many (a bundle costs what 32
+// lanes cost; the warp groups price a grid for 0.35 of a bundle's share in
+// mixed precision, 0.55 in FP64, so fewer go there).
+constexpr int kBundleMinMixed = 11;
+constexpr int kBundleMinF64 = 17;
+// A bundle takes 1.6 ms (mixed) or 2.4 ms (FP64) for 40 steps however few run
+// at once, which the warp groups beat on small batches: bundles where the
+// (N, precision) has at least this many Inner nodes per SM.  Measured
+// crossovers, in instances (nodes per SM): mixed N=3 level 5 550 (3 700), N=4
+// level 5 200 (3 400), N=6 level 6 20 (5 300), N=8 level 5 19 (4 000); FP64
+// N=3 level 5 310 (2 100), N=4 level 5 75 (1 250), N=6 level 5 10 (700).
+constexpr int64_t kBundleNodesMixed = 4000;
+constexpr int64_t kBundleNodesF64 = 1300;
 
 // Global-memory groups: at most this much scratch per launch class (it bounds
 // the number of resident blocks, each holding one grid's state).
@@ -291,6 +318,7 @@ struct Plan {
     std::vector<double> coefs;        // per grid, instance order
     std::vector<int8_t> levels;       // per grid (dim = 8 each), instance order
     std::vector<LaunchClass> classes;
+    std::vector<Bundle> bundles;      // per class, in the order of its items
     // device
     InstDev* d_insts = nullptr;
     Item* d_items = nullptr;
@@ -315,8 +343,23 @@ struct Plan {
         int64_t desc_offset = 0;  // into d_cdesc
     };
     std::vector<WarpLaunch> wl;
+    // bundle launches: one per (N, precision) over all its grid sizes
+    struct BundleLaunch {
+        int N = 0;
+        bool mixed = false;
+        std::vector<BundleClass> cls;
+        std::vector<int> covers;
+        int grid = 1, smem_warp = 0;
+        int lu_stride = 0;        // factor scratch per four warps of a block
+        int64_t desc_offset = 0;  // into d_bcls
+    };
+    std::vector<BundleLaunch> bl;
+    Bundle* d_bundles = nullptr;
+    BundleClass* d_bcls = nullptr;
     ClassDesc* d_cdesc = nullptr;
-    int64_t n_cdesc = 0;
+    int64_t n_cdesc = 0, n_bcls = 0;
+    unsigned char* d_blu = nullptr;  // factor scratch of the bundle launches (one after the other)
+    int64_t blu_len = 0, blu_cap = 0;
     bool use_multi = true;  // launch strategy (the autotuner may switch it)
     int glog_delta = 0;     // warp groups: lanes per grid widened by 2^glog_delta (autotuned)
     bool shared_u = false;  // d_u belongs to another plan (the FP64 re-solve writes there)
@@ -335,8 +378,14 @@ struct Plan {
         cudaFree(d_state);
         cudaFree(d_lu);
         cudaFree(d_cdesc);
+        cudaFree(d_bundles);
+        cudaFree(d_bcls);
+        cudaFree(d_blu);
+        d_blu = nullptr;
         d_lu = nullptr;
         d_cdesc = nullptr;
+        d_bundles = nullptr;
+        d_bcls = nullptr;
         d_insts = nullptr; d_items = nullptr; d_coefs = nullptr; d_u = nullptr;
         d_prices = nullptr; d_queue = nullptr; d_flag = nullptr; d_state = nullptr;
     }
@@ -352,7 +401,9 @@ int log2i(int v)
 // Host-side plan: validated instances, grid list grouped into launch classes
 // (largest grids first), launch shapes and the size of the line-solve scratch.
 // No device memory is touched.
-int plan_host(const amfrw_params* ps, int n, bool keep_state, Plan& P)
+// bundles: whether grids may be solved as bundles; bundle_scratch: whether those
+// may keep line-solve factors in global scratch.
+int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool bundle_scratch, Plan& P)
 {
     if (n < 1) return fail(AMFRW_EINVAL, "need at least one instance");
     if (!ps) return fail(AMFRW_EINVAL, "params is NULL");
@@ -481,6 +532,9 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, Plan& P)
     P.n_grids = (int)P.coefs.size();
     P.state_len = state_off;
     const int sms = num_sms();
+    int64_t warp_nodes[kMaxDim + 1][2] = {};  // Inner nodes of the warp-solved grids per (N, precision)
+    for (const Tmp& t : all)
+        if (t.warp) warp_nodes[t.N][t.mixed ? 1 : 0] += t.L;
     for (size_t k = 0; k < all.size();) {
         size_t e = k;
         int gmax = 0, lmax = 0;
@@ -533,7 +587,58 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, Plan& P)
             c.grid = (int)std::max<int64_t>(1, std::min<int64_t>(c.grid, kMemScratchBudget / c.lu_stride));
         c.lu_offset = P.lu_scratch_len;
         P.lu_scratch_len += c.lu_stride * c.grid;
-        for (size_t q = k; q < e; ++q) P.items.push_back(all[q].it);
+        c.bundle_begin = (int)P.bundles.size();
+        c.rest_begin = c.item_begin;
+        if (c.warp && bundles && warp_nodes[c.N][c.mixed ? 1 : 0] >= sms * (c.mixed ? kBundleNodesMixed : kBundleNodesF64)) {
+            // runs of equal levels (adjacent, in instance order): whole
+            // bundles of the instances with Neumann faces, then what is left
+            std::vector<Item> rest;
+            for (size_t r0 = k; r0 < e;) {
+                size_t r1 = r0;
+                std::vector<size_t> run;
+                for (; r1 < e && memcmp(all[r1].it.lv, all[r0].it.lv, sizeof(all[r0].it.lv)) == 0; ++r1) {
+                    if (P.insts[(size_t)all[r1].it.inst].bc == 0) run.push_back(r1);
+                    else rest.push_back(all[r1].it);
+                }
+                int take = (int)run.size() / kBundleLanes * kBundleLanes;
+                if ((int)run.size() - take >= (c.mixed ? kBundleMinMixed : kBundleMinF64)) take = (int)run.size();
+                if (take > 0) {
+                    const int nw = bundle_warps(lmax);
+                    int bytes = 0, lu = 0;
+                    for (int g : {c.glog, 5}) {  // (the widths the launches may give the class)
+                        const BundleLayout y = bundle_layout(c.N, all[r0].it.lv, c.mixed, g, 0);
+                        bytes = std::max(bytes, y.total);
+                        lu = std::max(lu, y.lu < 0 ? y.nlu : 0);
+                    }
+                    if (bytes > bundle_budget(c.mixed, lmax) || (lu > 0 && !bundle_scratch)) {
+                        take = 0;
+                    } else {
+                        c.bundle_smem = std::max(c.bundle_smem, (bytes / nw + 255) & ~255);
+                        c.bundle_lu = std::max(c.bundle_lu, lu);
+                    }
+                }
+                for (int q = 0; q < take; ++q) {
+                    if (q % kBundleLanes == 0)
+                        P.bundles.push_back(Bundle{(int32_t)P.items.size(), std::min(kBundleLanes, take - q)});
+                    P.items.push_back(all[run[(size_t)q]].it);
+                }
+                for (size_t q = (size_t)take; q < run.size(); ++q) rest.push_back(all[run[q]].it);
+                r0 = r1;
+            }
+            // bundles with the same inner block run the same code: next to each
+            // other they share the instruction caches
+            std::vector<std::pair<int, Bundle>> byp;
+            for (size_t q = (size_t)c.bundle_begin; q < P.bundles.size(); ++q)
+                byp.push_back({bundle_layout(c.N, P.items[(size_t)P.bundles[q].begin].lv, c.mixed, c.glog, 0).pat, P.bundles[q]});
+            std::stable_sort(byp.begin(), byp.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
+            for (size_t q = 0; q < byp.size(); ++q) P.bundles[(size_t)c.bundle_begin + q] = byp[q].second;
+            c.bundle_count = (int)P.bundles.size() - c.bundle_begin;
+            c.rest_begin = (int)P.items.size();
+            P.items.insert(P.items.end(), rest.begin(), rest.end());
+        } else {
+            for (size_t q = k; q < e; ++q) P.items.push_back(all[q].it);
+        }
+        c.rest_count = c.item_begin + c.item_count - c.rest_begin;
         P.classes.push_back(c);
         k = e;
     }
@@ -546,6 +651,8 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, Plan& P)
 int build_warp_launches(Plan& P)
 {
     P.wl.clear();
+    P.bl.clear();
+    std::vector<int> width(P.classes.size(), 0);  // log2 lanes of each class's warp groups
     const int smem_cap = max_smem_optin();
     const int sms = num_sms();
     std::vector<std::vector<int>> groups;
@@ -618,10 +725,15 @@ int build_warp_launches(Plan& P)
                 ++d.glog;
                 d.smem_group = group_smem(d.glog);
             }
+            width[(size_t)c] = d.glog;
+            if (L.rest_count == 0) continue;
+            d.item_begin = L.rest_begin;
+            d.item_count = L.rest_count;
             w.cls.push_back(d);
             w.smem_warp = std::max(w.smem_warp, d.smem_group << (5 - d.glog));
             items += d.item_count << d.glog;  // lanes of work
         }
+        if (w.cls.empty()) continue;
         if (w.smem_warp > smem_cap)
             return fail(AMFRW_ETOOBIG, "the work groups of one warp do not fit in shared memory");
         const int wpb = std::min(kWarpsPerBlock, std::max(1, smem_cap / w.smem_warp));
@@ -636,25 +748,84 @@ int build_warp_launches(Plan& P)
         P.wl.push_back(w);
     }
     P.n_cdesc = off;
+    // bundles: one launch per (N, precision), largest grids first
+    off = 0;
+    for (int N = 2; N <= kMaxDim; ++N) {
+        for (int mixed = 0; mixed < 2; ++mixed) {
+            Plan::BundleLaunch b;
+            b.N = N;
+            b.mixed = mixed != 0;
+            for (size_t c = 0; c < P.classes.size(); ++c) {
+                const LaunchClass& L = P.classes[c];
+                if (L.N != N || (int)L.mixed != mixed || L.bundle_count == 0) continue;
+                b.covers.push_back((int)c);
+                b.smem_warp = std::max(b.smem_warp, L.bundle_smem);
+                b.lu_stride = std::max(b.lu_stride, (L.bundle_lu + 255) & ~255);
+            }
+            if (b.covers.empty()) continue;
+            std::sort(b.covers.begin(), b.covers.end(), [&](int x, int y) {
+                return P.items[P.classes[x].item_begin].L > P.items[P.classes[y].item_begin].L;
+            });
+            int need = 0;  // warps of work
+            for (int c : b.covers) {
+                const LaunchClass& L = P.classes[(size_t)c];
+                BundleClass d{};
+                d.warps = bundle_warps(P.items[L.item_begin].L);
+                d.begin = L.bundle_begin;
+                d.count = L.bundle_count;
+                d.qidx = (int)P.classes.size() + c;
+                d.tlog = width[(size_t)c];
+                need += d.warps * d.count;
+                b.cls.push_back(d);
+            }
+            const size_t smem = (size_t)b.smem_warp * (kBundleThreads / 32);
+            const int per_sm = occ_for(N)(b.mixed, kBundle, kBundleThreads, smem);
+            if (per_sm < 1) return fail(AMFRW_ETOOBIG, "no resident block possible for a bundle launch");
+            b.grid = std::max(1, std::min((need + kBundleThreads / 32 - 1) / (kBundleThreads / 32), per_sm * sms));
+            b.desc_offset = off;
+            off += (int64_t)b.cls.size();
+            P.bl.push_back(b);
+        }
+    }
+    P.n_bcls = off;
+    P.blu_len = 0;
+    for (const Plan::BundleLaunch& b : P.bl) P.blu_len = std::max(P.blu_len, (int64_t)b.grid * 2 * b.lu_stride);
     return AMFRW_OK;
 }
 
 int upload_warp_launches(Plan& P)
 {
-    if (P.n_cdesc == 0) return AMFRW_OK;
     std::vector<ClassDesc> all;
     for (const Plan::WarpLaunch& w : P.wl) all.insert(all.end(), w.cls.begin(), w.cls.end());
-    if (!P.d_cdesc) CUDA_TRY(cudaMalloc(&P.d_cdesc, sizeof(ClassDesc) * all.size()));
-    CUDA_TRY(cudaMemcpyAsync(P.d_cdesc, all.data(), sizeof(ClassDesc) * all.size(),
-                             cudaMemcpyHostToDevice, P.stream));
-    // the upload must complete before `all` goes away
-    CUDA_TRY(cudaStreamSynchronize(P.stream));
+    std::vector<BundleClass> bc;
+    for (const Plan::BundleLaunch& b : P.bl) bc.insert(bc.end(), b.cls.begin(), b.cls.end());
+    // (room for one descriptor per class: the launches may be rebuilt)
+    const size_t nc = std::max<size_t>(1, P.classes.size());
+    if (!all.empty()) {
+        if (!P.d_cdesc) CUDA_TRY(cudaMalloc(&P.d_cdesc, sizeof(ClassDesc) * nc));
+        CUDA_TRY(cudaMemcpyAsync(P.d_cdesc, all.data(), sizeof(ClassDesc) * all.size(),
+                                 cudaMemcpyHostToDevice, P.stream));
+    }
+    if (!bc.empty()) {
+        if (!P.d_bcls) CUDA_TRY(cudaMalloc(&P.d_bcls, sizeof(BundleClass) * nc));
+        CUDA_TRY(cudaMemcpyAsync(P.d_bcls, bc.data(), sizeof(BundleClass) * bc.size(), cudaMemcpyHostToDevice, P.stream));
+    }
+    if (P.blu_len > P.blu_cap) {
+        if (P.d_blu) CUDA_TRY(cudaStreamSynchronize(P.stream));
+        cudaFree(P.d_blu);
+        P.d_blu = nullptr;
+        P.blu_cap = 0;
+        CUDA_TRY(cudaMalloc(&P.d_blu, (size_t)P.blu_len));
+        P.blu_cap = P.blu_len;
+    }
+    // the uploads must complete before the vectors go away
+    if (!all.empty() || !bc.empty()) CUDA_TRY(cudaStreamSynchronize(P.stream));
     return AMFRW_OK;
 }
 
-int build_plan(const amfrw_params* ps, int n, void* stream, bool keep_state, Plan& P)
+int build_plan(const amfrw_params* ps, int n, void* stream, bool keep_state, bool bundles, Plan& P)
 {
-    int st = plan_host(ps, n, keep_state, P);
+    int st = plan_host(ps, n, keep_state, bundles, true, P);
     if (st != AMFRW_OK) return st;
     CUDA_TRY(cudaGetDevice(&P.device));
     P.stream = (cudaStream_t)stream;
@@ -664,10 +835,15 @@ int build_plan(const amfrw_params* ps, int n, void* stream, bool keep_state, Pla
     CUDA_TRY(cudaMalloc(&P.d_coefs, sizeof(double) * P.coefs.size()));
     CUDA_TRY(cudaMalloc(&P.d_u, sizeof(double) * P.coefs.size()));
     CUDA_TRY(cudaMalloc(&P.d_prices, sizeof(double) * P.n_inst));
-    CUDA_TRY(cudaMalloc(&P.d_queue, sizeof(int32_t) * std::max<size_t>(1, P.classes.size())));
+    CUDA_TRY(cudaMalloc(&P.d_queue, sizeof(int32_t) * 2 * std::max<size_t>(1, P.classes.size())));
     CUDA_TRY(cudaMalloc(&P.d_flag, sizeof(int32_t)));
     if (keep_state) CUDA_TRY(cudaMalloc(&P.d_state, sizeof(double) * std::max<int64_t>(1, P.state_len)));
     if (P.lu_scratch_len > 0) CUDA_TRY(cudaMalloc(&P.d_lu, (size_t)P.lu_scratch_len));
+    if (!P.bundles.empty()) {
+        CUDA_TRY(cudaMalloc(&P.d_bundles, sizeof(Bundle) * P.bundles.size()));
+        CUDA_TRY(cudaMemcpyAsync(P.d_bundles, P.bundles.data(), sizeof(Bundle) * P.bundles.size(),
+                                 cudaMemcpyHostToDevice, P.stream));
+    }
     int st2 = build_warp_launches(P);
     if (st2 != AMFRW_OK) return st2;
     st2 = upload_warp_launches(P);
@@ -755,21 +931,25 @@ SolveArgs class_args(const Plan& P, const LaunchClass& L, int c, int steps, int 
     return a;
 }
 
-// The launches of one solve, in order: the warp-group launches, then the CTA
-// classes.  Each record is (warp launch index or -1, class index or -1).
-std::vector<std::pair<int, int>> launch_records(const Plan& P)
+// The launches of one solve, in order: the bundles, the warp groups, the CTA
+// classes.  Each record has one index of the three, the others -1.
+struct LaunchRec {
+    int bundle, warp, cls;
+};
+std::vector<LaunchRec> launch_records(const Plan& P)
 {
-    std::vector<std::pair<int, int>> r;
-    for (size_t w = 0; w < P.wl.size(); ++w) r.push_back({(int)w, -1});
+    std::vector<LaunchRec> r;
+    for (size_t b = 0; b < P.bl.size(); ++b) r.push_back({(int)b, -1, -1});
+    for (size_t w = 0; w < P.wl.size(); ++w) r.push_back({-1, (int)w, -1});
     for (size_t c = 0; c < P.classes.size(); ++c)
-        if (!P.classes[c].warp) r.push_back({-1, (int)c});
+        if (!P.classes[c].warp) r.push_back({-1, -1, (int)c});
     return r;
 }
 
 int run_solve(Plan& P, int steps, int flags, cudaEvent_t* ev = nullptr)
 {
-    CUDA_TRY(cudaMemsetAsync(P.d_queue, 0, sizeof(int32_t) * P.classes.size(), P.stream));
-    const std::vector<std::pair<int, int>> recs = launch_records(P);
+    CUDA_TRY(cudaMemsetAsync(P.d_queue, 0, sizeof(int32_t) * 2 * P.classes.size(), P.stream));
+    const std::vector<LaunchRec> recs = launch_records(P);
     // inside a graph capture the records are external, so that they also
     // record when the graph is replayed; outside they are plain records
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -778,8 +958,23 @@ int run_solve(Plan& P, int steps, int flags, cudaEvent_t* ev = nullptr)
     for (size_t r = 0; r < recs.size(); ++r) {
         int rc = 0;
         if (ev) CUDA_TRY(cudaEventRecordWithFlags(ev[2 * r], P.stream, rec_flags));
-        if (recs[r].first >= 0) {
-            const Plan::WarpLaunch& w = P.wl[recs[r].first];
+        if (recs[r].bundle >= 0) {
+            const Plan::BundleLaunch& b = P.bl[(size_t)recs[r].bundle];
+            BundleArgs a{};
+            a.items = P.d_items;
+            a.insts = P.d_insts;
+            a.bundles = P.d_bundles;
+            a.classes = P.d_bcls + b.desc_offset;
+            a.u_out = P.d_u;
+            a.queue = P.d_queue;
+            a.n_classes = (int32_t)b.cls.size();
+            a.steps = steps;
+            a.smem_warp = b.smem_warp;
+            a.lu_stride = b.lu_stride;
+            a.lu_scratch = P.d_blu;
+            rc = launch_bundle_for(b.N)(a, b.mixed, b.grid, (size_t)b.smem_warp * (kBundleThreads / 32), P.stream);
+        } else if (recs[r].warp >= 0) {
+            const Plan::WarpLaunch& w = P.wl[recs[r].warp];
             SolveArgs a = class_args(P, P.classes[w.covers[0]], 0, steps, flags);
             a.items = P.d_items;
             a.queue = P.d_queue;
@@ -788,7 +983,7 @@ int run_solve(Plan& P, int steps, int flags, cudaEvent_t* ev = nullptr)
             a.smem_warp = w.smem_warp;
             rc = launch_for(w.N)(a, w.mixed, kWarpGroup, w.block, w.grid, w.smem, P.stream);
         } else {
-            const int c = recs[r].second;
+            const int c = recs[r].cls;
             const LaunchClass& L = P.classes[c];
             rc = launch_for(L.N)(class_args(P, L, c, steps, flags), L.mixed, L.kind, L.block, L.grid,
                                  L.smem, P.stream);
@@ -1073,7 +1268,9 @@ int build_promotion(amfrw_batch* b, const amfrw_params* ps, int n, void* stream)
     b->promo.reset(new (std::nothrow) Plan());
     if (!b->promo) return fail(AMFRW_ENOMEM, "host allocation failed");
     Plan& Q = *b->promo;
-    int st = build_plan(q.data(), n, stream, false, Q);
+    // (no bundles: few instances are re-solved, and a bundle costs what its
+    // 32 lanes cost however few are marked)
+    int st = build_plan(q.data(), n, stream, false, false, Q);
     if (st != AMFRW_OK) return st;
     cudaFree(Q.d_u);
     Q.d_u = b->plan.d_u;
@@ -1092,7 +1289,7 @@ int build_promotion(amfrw_batch* b, const amfrw_params* ps, int n, void* stream)
 
 int ensure_events(amfrw_batch* b)
 {
-    const size_t need = 2 * b->plan.classes.size();
+    const size_t need = 2 * (b->plan.classes.size() + b->plan.bl.size());
     while (b->ev.size() < need) {
         cudaEvent_t e;
         CUDA_TRY(cudaEventCreate(&e));
@@ -1129,7 +1326,7 @@ int amfrw_problem_create(const amfrw_params* p, void* cuda_stream, amfrw_problem
     *out = nullptr;
     amfrw_problem* h = new (std::nothrow) amfrw_problem();
     if (!h) return fail(AMFRW_ENOMEM, "host allocation failed");
-    int st = build_plan(p, 1, cuda_stream, true, h->plan);
+    int st = build_plan(p, 1, cuda_stream, true, false, h->plan);
     if (st != AMFRW_OK) {
         delete h;
         return st;
@@ -1223,7 +1420,7 @@ int amfrw_batch_create(const amfrw_params* ps, int32_t n, void* cuda_stream, amf
     *out = nullptr;
     amfrw_batch* b = new (std::nothrow) amfrw_batch();
     if (!b) return fail(AMFRW_ENOMEM, "host allocation failed");
-    int st = build_plan(ps, n, cuda_stream, false, b->plan);
+    int st = build_plan(ps, n, cuda_stream, false, true, b->plan);
     if (st != AMFRW_OK) {
         delete b;
         return st;
@@ -1352,10 +1549,10 @@ int amfrw_batch_autotune(amfrw_batch* b, int32_t trials, int32_t* use_multi_out)
         // launch record of each CTA class
         std::vector<size_t> at;
         {
-            const std::vector<std::pair<int, int>> recs = launch_records(P);
+            const std::vector<LaunchRec> recs = launch_records(P);
             for (int c : cta)
                 for (size_t r = 0; r < recs.size(); ++r)
-                    if (recs[r].second == c) at.push_back(r);
+                    if (recs[r].cls == c) at.push_back(r);
         }
         float tot[2];
         std::vector<float> rec[2];
@@ -1446,19 +1643,23 @@ int amfrw_batch_kernel_times(amfrw_batch* b, float* ms_out, double* node_steps_o
     if (!b || !ms_out || !n_out) return fail(AMFRW_EINVAL, "NULL argument");
     if (b->ev.empty()) return fail(AMFRW_EINVAL, "timing is not enabled");
     const Plan& P = b->plan;
-    const std::vector<std::pair<int, int>> recs = launch_records(P);
+    const std::vector<LaunchRec> recs = launch_records(P);
     const int n = std::min<int>(cap, (int)recs.size());
     for (int r = 0; r < n; ++r) {
         CUDA_TRY(cudaEventSynchronize(b->ev[2 * r + 1]));
         CUDA_TRY(cudaEventElapsedTime(&ms_out[r], b->ev[2 * r], b->ev[2 * r + 1]));
         std::vector<int> cls;
-        if (recs[r].first >= 0) cls = P.wl[recs[r].first].covers;
-        else cls.push_back(recs[r].second);
+        if (recs[r].bundle >= 0) cls = P.bl[recs[r].bundle].covers;
+        else if (recs[r].warp >= 0) cls = P.wl[recs[r].warp].covers;
+        else cls.push_back(recs[r].cls);
         double s = 0.0;
         int dim = 0;
         for (int c : cls) {
             const LaunchClass& L = P.classes[c];
-            for (int k = L.item_begin; k < L.item_begin + L.item_count; ++k)
+            // a warp class's items are split between its bundles and its warp groups
+            const int k0 = recs[r].warp >= 0 ? L.rest_begin : L.item_begin;
+            const int k1 = recs[r].bundle >= 0 ? L.rest_begin : L.item_begin + L.item_count;
+            for (int k = k0; k < k1; ++k)
                 s += (double)P.items[k].L * (double)P.insts[P.items[k].inst].n_steps;
             dim = L.N;  // a launch's classes share N
         }
@@ -1474,7 +1675,7 @@ int amfrw_batch_io_bytes(const amfrw_batch* b, int64_t* h2d_bytes, int64_t* d2h_
     if (!b || !h2d_bytes || !d2h_bytes) return fail(AMFRW_EINVAL, "NULL argument");
     const Plan& P = b->plan;
     *h2d_bytes = (int64_t)(sizeof(InstDev) * P.insts.size() + sizeof(Item) * P.items.size() +
-                           sizeof(double) * P.coefs.size());
+                           sizeof(double) * P.coefs.size() + sizeof(Bundle) * P.bundles.size());
     *d2h_bytes = (int64_t)(sizeof(double) * P.n_inst + sizeof(int32_t));
     return AMFRW_OK;
 }
@@ -1677,15 +1878,24 @@ void noalloc_release_host(Plan& P)
     std::vector<int8_t>().swap(P.levels);
     std::vector<LaunchClass>().swap(P.classes);
     std::vector<Plan::WarpLaunch>().swap(P.wl);
+    std::vector<Bundle>().swap(P.bundles);
+    std::vector<Plan::BundleLaunch>().swap(P.bl);
     P.d_insts = nullptr; P.d_items = nullptr; P.d_coefs = nullptr; P.d_u = nullptr;
     P.d_prices = nullptr; P.d_queue = nullptr; P.d_flag = nullptr; P.d_state = nullptr;
     P.d_lu = nullptr;
     P.d_cdesc = nullptr;
+    P.d_bundles = nullptr;
+    P.d_bcls = nullptr;
+    P.d_blu = nullptr;
 }
 
-int noalloc_run(const amfrw_params* ps, int n, double* d_prices_out, cudaStream_t stream, Plan& P)
+// Status of a first plan whose bundle lists no longer fit the array: the call
+// plans again without bundles (which need no lists).
+constexpr int kNoallocRetry = -1;
+
+int noalloc_run(const amfrw_params* ps, int n, double* d_prices_out, cudaStream_t stream, bool bundles, Plan& P)
 {
-    int st = plan_host(ps, n, false, P);
+    int st = plan_host(ps, n, false, bundles, false, P);
     if (st == AMFRW_OK) st = build_warp_launches(P);
     if (st != AMFRW_OK) return st;
     const int s0 = P.insts[0].n_steps;
@@ -1697,9 +1907,11 @@ int noalloc_run(const amfrw_params* ps, int n, double* d_prices_out, cudaStream_
     const int64_t o_coef = align256(o_item + (int64_t)(sizeof(Item) * P.items.size()));
     const int64_t o_u = align256(o_coef + (int64_t)(sizeof(double) * P.coefs.size()));
     const int64_t o_queue = align256(o_u + (int64_t)(sizeof(double) * P.coefs.size()));
-    const int64_t o_flag = align256(o_queue + (int64_t)(sizeof(int32_t) * P.classes.size()));
+    const int64_t o_flag = align256(o_queue + (int64_t)(sizeof(int32_t) * 2 * P.classes.size()));
     const int64_t o_desc = align256(o_flag + (int64_t)sizeof(int32_t));
-    const int64_t o_lu = align256(o_desc + (int64_t)(sizeof(ClassDesc) * P.n_cdesc));
+    const int64_t o_bdl = align256(o_desc + (int64_t)(sizeof(ClassDesc) * P.n_cdesc));
+    const int64_t o_bcls = align256(o_bdl + (int64_t)(sizeof(Bundle) * P.bundles.size()));
+    const int64_t o_lu = align256(o_bcls + (int64_t)(sizeof(BundleClass) * P.n_bcls));
     // the per-block slices of the CTA and global-memory classes (factors,
     // states) take what the array has left: a class that wants more blocks
     // than fit runs fewer (each block pulls grids from the class's queue
@@ -1718,6 +1930,7 @@ int noalloc_run(const amfrw_params* ps, int n, double* d_prices_out, cudaStream_
         P.lu_scratch_len = off;
     }
     const int64_t total = o_lu + P.lu_scratch_len;
+    if (total > (int64_t)AMFRW_NOALLOC_SCRATCH_BYTES && !P.bundles.empty()) return kNoallocRetry;
     if (total > (int64_t)AMFRW_NOALLOC_SCRATCH_BYTES)
         return fail(AMFRW_ETOOBIG, "problem needs " + std::to_string(total) +
                                        " bytes of scratch; amfrw_solve_noalloc is limited to " +
@@ -1734,6 +1947,15 @@ int noalloc_run(const amfrw_params* ps, int n, double* d_prices_out, cudaStream_
     P.d_flag = reinterpret_cast<int32_t*>(base + o_flag);
     P.d_lu = P.lu_scratch_len > 0 ? base + o_lu : nullptr;
     P.d_cdesc = reinterpret_cast<ClassDesc*>(base + o_desc);
+    P.d_bundles = reinterpret_cast<Bundle*>(base + o_bdl);
+    P.d_bcls = reinterpret_cast<BundleClass*>(base + o_bcls);
+    std::vector<BundleClass> bcls;
+    for (const Plan::BundleLaunch& b : P.bl) bcls.insert(bcls.end(), b.cls.begin(), b.cls.end());
+    if (!bcls.empty()) {
+        CUDA_TRY(cudaMemcpyAsync(P.d_bcls, bcls.data(), sizeof(BundleClass) * bcls.size(), cudaMemcpyHostToDevice, stream));
+        CUDA_TRY(cudaMemcpyAsync(P.d_bundles, P.bundles.data(), sizeof(Bundle) * P.bundles.size(),
+                                 cudaMemcpyHostToDevice, stream));
+    }
     std::vector<ClassDesc> descs;
     for (const Plan::WarpLaunch& w : P.wl) descs.insert(descs.end(), w.cls.begin(), w.cls.end());
     if (!descs.empty())
@@ -1770,7 +1992,12 @@ extern "C" int amfrw_solve_noalloc(const amfrw_params* ps, int32_t n, double* d_
         return fail(AMFRW_EINVAL, "amfrw_solve_noalloc must not be called while its stream is being captured");
     alignas(Plan) unsigned char buf[sizeof(Plan)];
     Plan* P = new (buf) Plan();
-    const int st = noalloc_run(ps, n, d_prices_out, (cudaStream_t)cuda_stream, *P);
+    int st = noalloc_run(ps, n, d_prices_out, (cudaStream_t)cuda_stream, true, *P);
     noalloc_release_host(*P);
+    if (st == kNoallocRetry) {
+        P = new (buf) Plan();
+        st = noalloc_run(ps, n, d_prices_out, (cudaStream_t)cuda_stream, false, *P);
+        noalloc_release_host(*P);
+    }
     return st;
 }

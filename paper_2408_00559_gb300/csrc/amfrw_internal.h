@@ -1,5 +1,6 @@
 // Library-internal records shared by the host launcher and the kernels.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 
 #ifdef __CUDACC__
@@ -116,7 +117,8 @@ AMFRW_HD constexpr int shape_bytes(int N) { return align16(4 * (10 * N + 8)); }
 AMFRW_HD constexpr int meta_bytes(int N) { return shape_bytes(N) + align16((int)sizeof(ActAxes)); }
 constexpr int kMetaBytesMax = meta_bytes(kMaxDim);
 
-// Work-group kinds.  kWarpGroup: a grid of at most 64 Inner nodes on (part
+// Work-group kinds.  kBundle: grids of at most 64 Inner nodes of many
+// instances, one instance per lane.  kWarpGroup: a grid of at most 64 Inner nodes on (part
 // of) one warp, everything in shared memory.  kCtaGroup: one CTA per grid,
 // the grid in shared memory, line-solve factors in a global scratch slice.
 // kMemGroup: one CTA per grid with the whole grid state in its block's slice
@@ -125,6 +127,7 @@ constexpr int kMetaBytesMax = meta_bytes(kMaxDim);
 constexpr int kWarpGroup = 0;
 constexpr int kCtaGroup = 1;
 constexpr int kMemGroup = 2;
+constexpr int kBundle = 3;
 
 // Rows of a line per lane in a line solve: at most 2 for warp groups (grids of
 // at most 64 Inner nodes), at most 8 for FP64 CTA groups and 4 for
@@ -327,6 +330,227 @@ struct SolveArgs {
 constexpr int kLoadState = 1;
 constexpr int kStoreState = 2;
 
+// Bundles (amfrw_bundle.cuh): up to 32 grids of one shape, one instance per
+// lane, on a group of warps that share the nodes.
+constexpr int kBundleThreads = 256;
+constexpr int kBundleLanes = 32;
+AMFRW_HD int bundle_warps(int L) { return L >= 64 ? 8 : 4; }
+
+struct Bundle {
+    int32_t begin, count;  // its grids: consecutive items of equal levels
+};
+
+// Bundles of one grid size in a launch.  tlog: log2 lanes of the warp group
+// that would solve one of these grids (it fixes the mixed-precision line
+// solves' split, so both give the same prices).
+struct BundleClass {
+    int32_t warps, begin, count, qidx, tlog, pad;
+};
+
+struct BundleArgs {
+    const Item* items;
+    const InstDev* insts;
+    const Bundle* bundles;
+    const BundleClass* classes;
+    double* u_out;
+    int32_t* queue;
+    int32_t n_classes, steps;
+    int32_t smem_warp;  // dynamic shared bytes per warp
+    int32_t lu_stride;  // bytes of lu_scratch per half block
+    unsigned char* lu_scratch;
+};
+
+// Shared memory a bundle of W warps may take: two blocks per SM in mixed
+// precision, one in FP64 (whose pipe eight warps keep busy).
+constexpr int kBundleSmemMixed = 112 * 1024;
+constexpr int kBundleSmemF64 = 225 * 1024;
+AMFRW_HD int bundle_budget(bool mixed, int L)
+{
+    return ((mixed ? kBundleSmemMixed : kBundleSmemF64) / 8 * bundle_warps(L)) & ~255;
+}
+
+// Node patterns of a bundle's grid: how many rows of which axes, in axis order,
+// a thread holds in registers.  The F evaluation takes blocks of four nodes
+// (four rows of one axis, kPatSeg, or two axes of two rows), the directional
+// solves up to eight rows of consecutive axes.
+// (pat_nodes: nodes of a block of the F evaluation.)
+constexpr int kPat8 = 0, kPat42 = 1, kPat24 = 2, kPat222 = 3, kPat4 = 4, kPat22 = 5, kPat2 = 6, kPat1 = 7, kPatSeg = 8;
+AMFRW_HD int pat_nodes(int p) { return p == kPatSeg || p == kPat22 ? 4 : (p == kPat2 ? 2 : 1); }
+
+// A bundle's shared memory.  Values of T (float in mixed precision, double
+// otherwise) lie in rows of 32 lanes; entries below are row numbers in the
+// coefficient table (rows) or byte offsets.  q numbers the axes with more
+// than one row, in axis order (V, if among them, is last).
+struct BundleLayout {
+    int32_t L, Lr, n, nr;             // nodes, rate nodes, axes, rate axes
+    int32_t pat, in[2];               // inner block: pattern, its axes q
+    int32_t ax[6], M[6], sh[6];       // axis number, rows, bit offset of its index in storage order
+    int32_t qd[6], qds[6], qpw[6];    // second-difference coefficients (row stride 0: one for all), outer coefficients
+    int32_t qns[6];                   // stride of the axis in the rate grid (V: 0)
+    int32_t cx[6][6], dr[6];          // pair coefficients, drift coefficients (-1: none)
+    int32_t ntab, cv, c0;             // rows: build_tables' tables; c_V; (FP64) centre coefficients
+    int32_t vsh, vmask;               // V's index in storage order
+    // the directional solves of a stage: groups of consecutive axes with at
+    // most eight rows together (pattern, first q, blocks, base nodes in blk),
+    // or one longer axis (pattern -1)
+    int32_t ng, gpat[6], gq[6], gv[6], gn[6], gblk[6];
+    int32_t luoff[6];                 // rows of an axis's line-solve factors
+    int32_t prog, pblk;               // block programs: offset, bytes per block
+    int32_t lu, nlu;                  // factors: offset (-1: in global scratch), bytes
+    int32_t blk, tab, H, red, Z, ZZ, K1, Kw, R;
+    int32_t cst, tabd, pay, scr;      // setup only, in the vectors' memory
+    int32_t total;
+};
+
+AMFRW_HD BundleLayout bundle_layout(int N, const int8_t* lv, bool mixed, int tlog, int base)
+{
+    BundleLayout y{};
+    const int rb = mixed ? 128 : 256;
+    int sh = 0, sumM = 0, npay = 0, longM = 1;
+    int bits[6] = {0, 0, 0, 0, 0, 0}, toff = 0;
+    for (int i = 0; i < N; ++i) {
+        if (lv[i] > 0) {
+            const int q = y.n++;
+            y.ax[q] = i;
+            y.M[q] = 1 << lv[i];
+            bits[q] = lv[i];
+            y.qns[q] = i < N - 1 ? 1 << sh : 0;
+            y.qd[q] = toff;
+            y.qds[q] = 1;
+            y.qpw[q] = toff + y.M[q];
+            if (i < N - 1) ++y.nr;
+        }
+        if (i < N - 1) {
+            sumM += 1 << lv[i];
+            npay += (1 << lv[i]) + 1;
+            toff += 3 << lv[i];
+        }
+        sh += lv[i];
+    }
+    const int MV = 1 << lv[N - 1], tlg = sh;
+    y.L = 1 << sh;
+    y.Lr = y.L >> lv[N - 1];
+    // the inner block: rates if they can fill it, V only when they cannot; an
+    // axis of four rows before a longer one, whose blocks have neighbours
+    y.pat = kPat1;
+    y.in[0] = y.in[1] = -1;
+    for (int pass = 0; pass < 2 && y.pat == kPat1; ++pass) {
+        const int m = pass == 0 ? y.nr : y.n;
+        int one[6], n1 = 0, seg = -1;
+        for (int q = 0; q < m; ++q) {
+            if (bits[q] == 1) one[n1++] = q;
+            else if (seg < 0 || bits[q] < bits[seg]) seg = q;
+        }
+        if (seg >= 0) {
+            y.pat = kPatSeg;
+            y.in[0] = seg;
+        } else if (n1 >= 2) {
+            y.pat = kPat22;
+            y.in[0] = one[0];
+            y.in[1] = one[1];
+        } else if (pass == 1 && n1 == 1) {
+            y.pat = kPat2;
+            y.in[0] = one[0];
+        }
+    }
+    const int ni = y.pat == kPat22 ? 2 : (y.pat == kPat1 ? 0 : 1);
+    sh = 0;
+    for (int a = 0; a < ni; ++a) {
+        y.sh[y.in[a]] = sh;
+        sh += bits[y.in[a]];
+    }
+    for (int q = 0; q < y.n; ++q) {
+        if (q == y.in[0] || q == y.in[1]) continue;
+        y.sh[q] = sh;
+        sh += bits[q];
+    }
+    const bool vact = y.n > y.nr;
+    y.vsh = vact ? y.sh[y.n - 1] : 0;
+    y.vmask = MV - 1;
+    // coefficient rows
+    int rows = 3 * sumM + MV;
+    y.ntab = rows;
+    y.cv = rows++;
+    if (vact) {
+        y.qd[y.n - 1] = y.cv;
+        y.qds[y.n - 1] = 0;
+    }
+    if (!mixed) {
+        y.c0 = rows;
+        rows += y.Lr;
+    }
+    for (int q = 0; q < y.n; ++q) {
+        y.dr[q] = -1;
+        if (q >= y.nr) continue;
+        for (int r = q + 1; r < y.n; ++r) {
+            y.cx[q][r] = rows;
+            rows += r < y.nr ? y.M[r] : 1;
+        }
+        if (y.ax[q] >= 1) {
+            y.dr[q] = rows;
+            rows += y.M[q] * y.qns[q];
+        }
+    }
+    // line-solve factors: the sizes of make_shape's (mixed precision), three
+    // values a row (FP64); the folded single-row axes have none
+    int nlu = 0, nblk = 0;
+    for (int q = 0; q < y.n; ++q) {
+        const int M = y.M[q], r = (q < y.nr ? MV : 1) * M;
+        const bool dense = mixed && M <= kDenseMaxRows;
+        if (dense) nlu = (nlu + 3) & ~3;
+        y.luoff[q] = nlu;
+        if (dense) nlu += r * M;
+        else if (mixed) nlu += r * lu_row_values(lanes_log(bits[q], tlg, tlog, kRowsLogWarp));
+        else nlu += r * 3;
+        if (M > kDenseMaxRows && M > longM) longM = M;
+    }
+    if (y.n == 0) nlu = 3;
+    for (int q = 0; q < y.n;) {
+        const int g = y.ng++;
+        y.gq[g] = q;
+        int b = bits[q], e = q + 1;
+        if (b > 3) {
+            y.gpat[g] = -1;
+        } else {
+            while (e < y.n && b + bits[e] <= 3) b += bits[e++];
+            y.gpat[g] = b == 3 ? (e - q == 1 ? kPat8 : (e - q == 3 ? kPat222 : (bits[q] == 2 ? kPat42 : kPat24)))
+                               : (b == 2 ? (e - q == 1 ? kPat4 : kPat22) : kPat2);
+            y.gn[g] = y.L >> b;
+            y.gblk[g] = nblk;
+            nblk += y.gn[g];
+        }
+        y.gv[g] = vact && e == y.n && e - q > 1 ? 1 : 0;  // V and rates in one group
+        q = e;
+    }
+    int o = base + align16((int)sizeof(BundleLayout)) + shape_bytes(N);
+    y.blk = o;    o = align16(o + 2 * nblk);
+    y.pblk = 16 * (2 + 2 * y.n + y.n * (y.n - 1));
+    y.prog = o;   o += y.pblk * (y.L / pat_nodes(y.pat));
+    y.tab = o;    o += rb * rows;
+    y.H = o;      o += rb * y.Lr;
+    y.red = o;    o += 256 * bundle_warps(y.L);
+    y.nlu = rb * nlu;
+    int x = o;
+    // (mixed precision: a block of zeros behind each vector the stencil reads,
+    // for Outer neighbours)
+    const int Lz = y.L + (mixed ? 4 : 0);
+    y.Z = x;      x += 256 * y.L;
+    y.ZZ = x;     x += mixed ? 256 * Lz : 0;
+    y.K1 = x;     x += rb * Lz;
+    y.Kw = x;     x += rb * Lz;
+    y.R = x;      x += rb * y.L;
+    int p = o;
+    y.cst = p;    p += rb * (int)(sizeof(Consts<float>) / sizeof(float));
+    y.tabd = p;   p += mixed ? 256 * y.ntab : 0;
+    y.pay = p;    p += 256 * 2 * npay;
+    y.scr = p;    p += mixed ? 128 * 6 * longM : 0;
+    // the factors last, in global scratch when they do not fit
+    o = x > p ? x : p;
+    y.lu = o - base + y.nlu <= bundle_budget(mixed, y.L) ? o : -1;
+    y.total = (o + (y.lu < 0 ? 0 : y.nlu) - base + 255) & ~255;
+    return y;
+}
+
 // Host-side launchers, one translation unit per dimension N.
 using LaunchFn = int (*)(const SolveArgs&, bool mixed, int kind, int block, int grid,
                          size_t smem, void* stream);
@@ -337,6 +561,14 @@ int launch_n5(const SolveArgs&, bool, int, int, int, size_t, void*);
 int launch_n6(const SolveArgs&, bool, int, int, int, size_t, void*);
 int launch_n7(const SolveArgs&, bool, int, int, int, size_t, void*);
 int launch_n8(const SolveArgs&, bool, int, int, int, size_t, void*);
+int launch_bundle_n2(const BundleArgs&, bool, int, size_t, void*);
+int launch_bundle_n3(const BundleArgs&, bool, int, size_t, void*);
+int launch_bundle_n4(const BundleArgs&, bool, int, size_t, void*);
+int launch_bundle_n5(const BundleArgs&, bool, int, size_t, void*);
+int launch_bundle_n6(const BundleArgs&, bool, int, size_t, void*);
+int launch_bundle_n7(const BundleArgs&, bool, int, size_t, void*);
+int launch_bundle_n8(const BundleArgs&, bool, int, size_t, void*);
+using BundleFn = int (*)(const BundleArgs&, bool mixed, int grid, size_t smem, void* stream);
 // Occupancy query for the same instantiation (blocks per SM).
 int occupancy(int N, bool mixed, int kind, int block, size_t smem);
 using OccFn = int (*)(bool mixed, int kind, int block, size_t smem);

@@ -1,3 +1,3 @@
 // Solver kernels for N = 5 axes (4 forward rate(s) and V).
-#include "amfrw_solver.cuh"
+#include "amfrw_bundle.cuh"
 AMFRW_INSTANTIATE(5)

@@ -1,3 +1,3 @@
 // Solver kernels for N = 8 axes (7 forward rate(s) and V).
-#include "amfrw_solver.cuh"
+#include "amfrw_bundle.cuh"
 AMFRW_INSTANTIATE(8)

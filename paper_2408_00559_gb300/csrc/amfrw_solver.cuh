@@ -51,6 +51,15 @@ constexpr double kQ21 = -4.0 / 3.0;
 constexpr double kB1 = 5.0 / 4.0;
 constexpr double kB2 = 3.0 / 4.0;
 
+// A grid's constants (Consts<T>) as an array of T, for the setup functions
+// that serve one grid per group (ST = 1) or one grid per lane, value q of
+// lane l at q * 32 + l (ST = 32, the pointer already advanced by the lane).
+constexpr int kOffRm = 4, kOffRh = kOffRm + kMaxDim * (kMaxDim - 1) / 2;
+constexpr int kOffSm = kOffRh + kMaxDim * (kMaxDim + 1) / 2, kOffG2 = kOffSm + kMaxDim;
+constexpr int kConstCount = kOffG2 + kMaxDim;
+static_assert(sizeof(Consts<float>) == sizeof(float) * kConstCount && sizeof(Consts<double>) == sizeof(double) * kConstCount,
+              "Consts is an array of its values");
+
 template <int N>
 struct Shape {
     int lv[N], M[N], sh[N], Sp[N];
@@ -281,26 +290,26 @@ __device__ __forceinline__ TC stencil_acc(const Shape<N>& s, const int (&j)[N], 
 // payoff_at: every value is bitwise the one payoff_at gives (second
 // differences over fine axes amplify any rounding difference by 1/h^2), at a
 // fraction of the cost.
-template <int N>
+template <int N, int ST = 1>
 __device__ __noinline__ double payoff_H(const Shape<N>& s, const double* pay, int payoff, const int (&j)[N],
-                                        const double* __restrict__ tab, const Consts<double>& c)
+                                        const double* __restrict__ tab, const double* __restrict__ cst)
 {
     constexpr int n = N - 1;  // rate axes
     const double* A = pay;
-    const double* Bv = pay + s.phalf;
+    const double* Bv = pay + s.phalf * ST;
     if (payoff == 0) {  // caplet: G = (F_1 - K)^+ depends on rate 1 only
         const int o = s.poff[0] + j[0];
-        const double x0 = fmax(A[o], 0.0);
-        const double m = fmax(A[o - 1], 0.0);
-        const double p = (j[0] == s.nf[0]) ? m : fmax(A[o + 1], 0.0);
-        return tab[s.toff[0] + j[0] - 1] * ((p - x0) - (x0 - m));
+        const double x0 = fmax(A[o * ST], 0.0);
+        const double m = fmax(A[(o - 1) * ST], 0.0);
+        const double p = (j[0] == s.nf[0]) ? m : fmax(A[(o + 1) * ST], 0.0);
+        return tab[(s.toff[0] + j[0] - 1) * ST] * ((p - x0) - (x0 - m));
     }
     double a[n], b[n], P0[n], S0[n];  // P0[r], S0[r]: product and sum before rate r
     double P = 1.0, S = 0.0;
 #pragma unroll
     for (int r = 0; r < n; ++r) {
-        a[r] = A[s.poff[r] + j[r]];
-        b[r] = Bv[s.poff[r] + j[r]];
+        a[r] = A[(s.poff[r] + j[r]) * ST];
+        b[r] = Bv[(s.poff[r] + j[r]) * ST];
         P0[r] = P;
         S0[r] = S;
         P *= b[r];
@@ -309,14 +318,14 @@ __device__ __noinline__ double payoff_H(const Shape<N>& s, const double* pay, in
     const double x0 = fmax(S, 0.0);
     // payoff with rate i at table offset oi (and rate k > i at ok; k < 0: none)
     auto g = [&](int i, int oi, int k, int ok) {
-        double p = P0[i] * Bv[oi];
-        double q = fma(A[oi], p, S0[i]);
+        double p = P0[i] * Bv[oi * ST];
+        double q = fma(A[oi * ST], p, S0[i]);
 #pragma unroll
         for (int r = 0; r < n; ++r) {
             if (r <= i) continue;
             const bool ch = r == k;
-            p *= ch ? Bv[ok] : b[r];
-            q = fma(ch ? A[ok] : a[r], p, q);
+            p *= ch ? Bv[ok * ST] : b[r];
+            q = fma(ch ? A[ok * ST] : a[r], p, q);
         }
         return fmax(q, 0.0);
     };
@@ -334,7 +343,7 @@ __device__ __noinline__ double payoff_H(const Shape<N>& s, const double* pay, in
     }
     double acc = 0.0;
 #pragma unroll
-    for (int i = 0; i < n; ++i) acc += tab[s.toff[i] + j[i] - 1] * lap[i];
+    for (int i = 0; i < n; ++i) acc += tab[(s.toff[i] + j[i] - 1) * ST] * lap[i];
 #pragma unroll
     for (int i = 0; i < n; ++i) {
         double inner = 0.0;
@@ -349,17 +358,17 @@ __device__ __noinline__ double payoff_H(const Shape<N>& s, const double* pay, in
                     const double mp = g(i, oi - 1, k, ok + 1);
                     const double mm = g(i, oi - 1, k, ok - 1);
                     const double mix = (pp - pm) - (mp - mm);
-                    inner += c.rm[upair(i, k)] * tab[s.toff[k] + s.M[k] + j[k] - 1] * mix;
+                    inner += cst[(kOffRm + upair(i, k)) * ST] * tab[(s.toff[k] + s.M[k] + j[k] - 1) * ST] * mix;
                 }
             }
         }
         if (i >= 1) {  // drift of rates 2..N-1 (eq. coef_adv), sum over rates 2..i
             double Sd = 0.0;
 #pragma unroll
-            for (int r = 1; r <= i; ++r) Sd += c.rh[ltri(i, r)] * tab[s.toff[r] + 2 * s.M[r] + j[r] - 1];
-            inner += Sd * c.g2[i] * grad[i];
+            for (int r = 1; r <= i; ++r) Sd += cst[(kOffRh + ltri(i, r)) * ST] * tab[(s.toff[r] + 2 * s.M[r] + j[r] - 1) * ST];
+            inner += Sd * cst[(kOffG2 + i) * ST] * grad[i];
         }
-        acc += tab[s.toff[i] + s.M[i] + j[i] - 1] * inner;
+        acc += tab[(s.toff[i] + s.M[i] + j[i] - 1) * ST] * inner;
     }
     return acc;
 }
@@ -374,26 +383,26 @@ __device__ __noinline__ double payoff_H(const Shape<N>& s, const double* pay, in
 // U_ik = sum_{i<m<k} a_m prod_{i<l<=m} b_l built up as k grows.  The sums are
 // associated differently from payoff_at, which moves H by a few ulps: far
 // below the FP32 rounding of the mode, and not used by the FP64 mode.
-template <int N>
+template <int N, int ST = 1>
 __device__ __noinline__ float payoff_H_fast(const Shape<N>& s, const double* pay, int payoff, const int (&j)[N],
-                                            const float* __restrict__ tab, const Consts<float>& c)
+                                            const float* __restrict__ tab, const float* __restrict__ cst)
 {
     constexpr int n = N - 1;  // rate axes
     const double* A = pay;
     if (payoff == 0) {  // caplet: G = (F_1 - K)^+ depends on rate 1 only
         const int o = s.poff[0] + j[0];
-        const double x0 = fmax(A[o], 0.0);
-        const double m = fmax(A[o - 1], 0.0);
-        const double p = (j[0] == s.nf[0]) ? m : fmax(A[o + 1], 0.0);
-        return tab[s.toff[0] + j[0] - 1] * (float)((p - x0) - (x0 - m));
+        const double x0 = fmax(A[o * ST], 0.0);
+        const double m = fmax(A[(o - 1) * ST], 0.0);
+        const double p = (j[0] == s.nf[0]) ? m : fmax(A[(o + 1) * ST], 0.0);
+        return tab[(s.toff[0] + j[0] - 1) * ST] * (float)((p - x0) - (x0 - m));
     }
-    const double* Bv = pay + s.phalf;
+    const double* Bv = pay + s.phalf * ST;
     double a[n], b[n], P0[n], S0[n], T[n + 1];
     double P = 1.0, S = 0.0;
 #pragma unroll
     for (int r = 0; r < n; ++r) {
-        a[r] = A[s.poff[r] + j[r]];
-        b[r] = Bv[s.poff[r] + j[r]];
+        a[r] = A[(s.poff[r] + j[r]) * ST];
+        b[r] = Bv[(s.poff[r] + j[r]) * ST];
         P0[r] = P;
         S0[r] = S;
         P *= b[r];
@@ -409,8 +418,8 @@ __device__ __noinline__ float payoff_H_fast(const Shape<N>& s, const double* pay
     for (int i = 0; i < n; ++i) {
         const int o = s.poff[i] + j[i];
         const bool top = j[i] == s.nf[i];
-        const double m = fmax(fma(P0[i] * Bv[o - 1], A[o - 1] + T[i + 1], S0[i]), 0.0);
-        const double p = top ? m : fmax(fma(P0[i] * Bv[o + 1], A[o + 1] + T[i + 1], S0[i]), 0.0);
+        const double m = fmax(fma(P0[i] * Bv[(o - 1) * ST], A[(o - 1) * ST] + T[i + 1], S0[i]), 0.0);
+        const double p = top ? m : fmax(fma(P0[i] * Bv[(o + 1) * ST], A[(o + 1) * ST] + T[i + 1], S0[i]), 0.0);
         const double dp = p - x0;
         const double dm = x0 - m;
         lap[i] = (float)(dp - dm);
@@ -418,7 +427,7 @@ __device__ __noinline__ float payoff_H_fast(const Shape<N>& s, const double* pay
     }
     float acc = 0.f;
 #pragma unroll
-    for (int i = 0; i < n; ++i) acc += tab[s.toff[i] + j[i] - 1] * lap[i];
+    for (int i = 0; i < n; ++i) acc += tab[(s.toff[i] + j[i] - 1) * ST] * lap[i];
     int kend = -1;  // the last rate off its upper face: no cross term lies beyond it
 #pragma unroll
     for (int k = 0; k < n; ++k)
@@ -430,22 +439,22 @@ __device__ __noinline__ float payoff_H_fast(const Shape<N>& s, const double* pay
             const int oi = s.poff[i] + j[i];
             // a corner's payoff is S0[i] + c (a_i' + w) with c = P0[i] b_i' of
             // rate i's neighbour row: S0[i] + c a_i' is formed once per rate i
-            const double cp = P0[i] * Bv[oi + 1], cm = P0[i] * Bv[oi - 1];
-            const double sp = fma(cp, A[oi + 1], S0[i]), sm = fma(cm, A[oi - 1], S0[i]);
+            const double cp = P0[i] * Bv[(oi + 1) * ST], cm = P0[i] * Bv[(oi - 1) * ST];
+            const double sp = fma(cp, A[(oi + 1) * ST], S0[i]), sm = fma(cm, A[(oi - 1) * ST], S0[i]);
             double Q = 1.0, U = 0.0;  // Q_ik, U_ik for the current k
 #pragma unroll
             for (int k = i + 1; k < n; ++k) {
                 if (k > kend) break;
                 if (j[k] != s.nf[k]) {
                     const int ok = s.poff[k] + j[k];
-                    const double wp = U + Q * Bv[ok + 1] * (A[ok + 1] + T[k + 1]);
-                    const double wm = U + Q * Bv[ok - 1] * (A[ok - 1] + T[k + 1]);
+                    const double wp = U + Q * Bv[(ok + 1) * ST] * (A[(ok + 1) * ST] + T[k + 1]);
+                    const double wm = U + Q * Bv[(ok - 1) * ST] * (A[(ok - 1) * ST] + T[k + 1]);
                     const double pp = fmax(fma(cp, wp, sp), 0.0);
                     const double pm = fmax(fma(cp, wm, sp), 0.0);
                     const double mp = fmax(fma(cm, wp, sm), 0.0);
                     const double mm = fmax(fma(cm, wm, sm), 0.0);
                     const float mix = (float)((pp - pm) - (mp - mm));
-                    inner += c.rm[upair(i, k)] * tab[s.toff[k] + s.M[k] + j[k] - 1] * mix;
+                    inner += cst[(kOffRm + upair(i, k)) * ST] * tab[(s.toff[k] + s.M[k] + j[k] - 1) * ST] * mix;
                 }
                 Q *= b[k];
                 U = fma(a[k], Q, U);
@@ -454,10 +463,10 @@ __device__ __noinline__ float payoff_H_fast(const Shape<N>& s, const double* pay
         if (i >= 1) {  // drift of rates 2..N-1 (eq. coef_adv), sum over rates 2..i
             float Sd = 0.f;
 #pragma unroll
-            for (int r = 1; r <= i; ++r) Sd += c.rh[ltri(i, r)] * tab[s.toff[r] + 2 * s.M[r] + j[r] - 1];
-            inner += Sd * c.g2[i] * grad[i];
+            for (int r = 1; r <= i; ++r) Sd += cst[(kOffRh + ltri(i, r)) * ST] * tab[(s.toff[r] + 2 * s.M[r] + j[r] - 1) * ST];
+            inner += Sd * cst[(kOffG2 + i) * ST] * grad[i];
         }
-        acc += tab[s.toff[i] + s.M[i] + j[i] - 1] * inner;
+        acc += tab[(s.toff[i] + s.M[i] + j[i] - 1) * ST] * inner;
     }
     return acc;
 }
@@ -619,15 +628,14 @@ __device__ __forceinline__ T shfl(T v, int src, int width, unsigned mask)
 }
 
 // Row r of (I - nu dt A_axis) for line class cls: lower a, diagonal b, upper c.
-template <int N>
-__device__ __forceinline__ void matrix_row(const Shape<N>& s, const double* tabd,
-                                           const Consts<double>& c, int axis, int cls, int r,
-                                           double& a, double& b, double& u)
+template <int N, int ST = 1>
+__device__ __forceinline__ void matrix_row(const Shape<N>& s, const double* tabd, double cV, double nudt,
+                                           int axis, int cls, int r, double& a, double& b, double& u)
 {
     const int M = s.M[axis];
-    const double delta = (axis < N - 1) ? tabd[s.toff[axis] + r] * tabd[s.toff[N - 1] + cls]
-                                        : c.cV * tabd[s.toff[N - 1] + r];
-    const double nd = c.nudt * delta;
+    const double delta = (axis < N - 1) ? tabd[(s.toff[axis] + r) * ST] * tabd[(s.toff[N - 1] + cls) * ST]
+                                        : cV * tabd[(s.toff[N - 1] + r) * ST];
+    const double nd = nudt * delta;
     if ((s.dmask >> axis) & 1) {
         // eq. bound1_0: rows 0..M-2 are the M-1 Inner nodes (no super-diagonal
         // in the last, whose upper neighbour holds Dirichlet data); row M-1 is
@@ -653,16 +661,16 @@ __device__ __forceinline__ void matrix_row(const Shape<N>& s, const double* tabd
 // axis, or, when V has one row too (then every b_i is a constant), the last
 // rate axis with more than one row.  This returns that product for row r of
 // line class cls of the target axis.
-template <int N>
-__device__ __forceinline__ double fold_scale(const Shape<N>& s, const double* tabd,
-                                             const Consts<double>& c, int axis, int cls, int r)
+template <int N, int ST = 1>
+__device__ __forceinline__ double fold_scale(const Shape<N>& s, const double* tabd, double cV, double nudt,
+                                             int axis, int cls, int r)
 {
     const int v = (axis == N - 1) ? r : cls;  // V index of the row
     double f = 1.0;
 #pragma unroll
     for (int i = 0; i < N - 1; ++i)  // (a Dirichlet axis of one row has no Inner node: identity)
-        if (((s.skip & ~s.dmask) >> i) & 1) f *= 1.0 + 2.0 * (c.nudt * (tabd[s.toff[i]] * tabd[s.toff[N - 1] + v]));
-    if ((s.skip >> (N - 1)) & 1) f *= 1.0 + 2.0 * (c.nudt * (c.cV * tabd[s.toff[N - 1]]));
+        if (((s.skip & ~s.dmask) >> i) & 1) f *= 1.0 + 2.0 * (nudt * (tabd[s.toff[i] * ST] * tabd[(s.toff[N - 1] + v) * ST]));
+    if ((s.skip >> (N - 1)) & 1) f *= 1.0 + 2.0 * (nudt * (cV * tabd[s.toff[N - 1] * ST]));
     return f;
 }
 
@@ -699,9 +707,9 @@ __device__ void pcr_setup(const Shape<N>& s, const double* tabd, const Consts<do
             for (int q = 0; q < RMAX; ++q) {
                 if (q < R) {
                     double ad, bd, ud;
-                    matrix_row<N>(s, tabd, c, axis, cl, p + P * q, ad, bd, ud);
+                    matrix_row<N>(s, tabd, c.cV, c.nudt, axis, cl, p + P * q, ad, bd, ud);
                     if (axis == s.last && s.skip) {  // the folded single-row solves
-                        const double f = fold_scale<N>(s, tabd, c, axis, cl, p + P * q);
+                        const double f = fold_scale<N>(s, tabd, c.cV, c.nudt, axis, cl, p + P * q);
                         ad *= f;
                         bd *= f;
                         ud *= f;
@@ -866,9 +874,9 @@ struct NoEpi {
 // sums at most 1), and solves for the M unit vectors.  Entry (q, col) is
 // stored in row q at position q XOR col, the order in which dense_mix meets
 // the rows of a line.
-template <int N>
-__device__ __noinline__ void dense_setup(const Shape<N>& s, const double* tabd, const Consts<double>& c, float* lu,
-                            int rank, int gsize)
+template <int N, int ST = 1>
+__device__ __noinline__ void dense_setup(const Shape<N>& s, const double* tabd, double cV, double nudt,
+                                         float* lu, int rank, int gsize)
 {
     int total = 0;  // (axis, class) pairs of the dense axes
 #pragma unroll
@@ -885,16 +893,16 @@ __device__ __noinline__ void dense_setup(const Shape<N>& s, const double* tabd, 
         const int M = s.M[axis];
         const bool fold = axis == s.last && s.skip;
         // a rate axis's fold product depends on its class (the V index) only
-        const double fr = (fold && axis < N - 1) ? fold_scale<N>(s, tabd, c, axis, cls, 0) : 1.0;
+        const double fr = (fold && axis < N - 1) ? fold_scale<N, ST>(s, tabd, cV, nudt, axis, cls, 0) : 1.0;
         float lo[kDenseMaxRows], inv[kDenseMaxRows], gam[kDenseMaxRows];
         float gp = 0.f;
 #pragma unroll
         for (int q = 0; q < kDenseMaxRows; ++q) {
             if (q < M) {
                 double ad, bd, ud;
-                matrix_row<N>(s, tabd, c, axis, cls, q, ad, bd, ud);
+                matrix_row<N, ST>(s, tabd, cV, nudt, axis, cls, q, ad, bd, ud);
                 if (fold) {
-                    const double f = (axis < N - 1) ? fr : fold_scale<N>(s, tabd, c, axis, cls, q);
+                    const double f = (axis < N - 1) ? fr : fold_scale<N, ST>(s, tabd, cV, nudt, axis, cls, q);
                     ad *= f;
                     bd *= f;
                     ud *= f;
@@ -905,7 +913,7 @@ __device__ __noinline__ void dense_setup(const Shape<N>& s, const double* tabd, 
                 gam[q] = gp;
             }
         }
-        float* out = lu + s.luoff[axis] + cls * M * M;
+        float* out = lu + (s.luoff[axis] + cls * M * M) * ST;
 #pragma unroll 1
         for (int col = 0; col < M; ++col) {
             // forward elimination into the output slots, then back substitution there
@@ -914,14 +922,14 @@ __device__ __noinline__ void dense_setup(const Shape<N>& s, const double* tabd, 
             for (int q = 0; q < kDenseMaxRows; ++q) {
                 if (q < M) {
                     yp = ((q == col ? 1.f : 0.f) - lo[q] * yp) * inv[q];
-                    out[q * M + (q ^ col)] = yp;
+                    out[(q * M + (q ^ col)) * ST] = yp;
                 }
             }
             float x = 0.f;  // the last row has no upper neighbour (gam = 0 there)
 #pragma unroll
             for (int q = kDenseMaxRows - 1; q >= 0; --q) {
                 if (q < M) {
-                    float& o = out[q * M + (q ^ col)];
+                    float& o = out[(q * M + (q ^ col)) * ST];
                     x = o - gam[q] * x;
                     o = x;
                 }
@@ -1025,7 +1033,7 @@ __device__ void pcr_setup_mem(const Shape<N>& s, const double* tabd, const Const
             if (act)
                 for (int q = 0; q < R; ++q) {
                     double a, b, u;
-                    matrix_row<N>(s, tabd, c, axis, cl, p + P * q, a, b, u);
+                    matrix_row<N>(s, tabd, c.cV, c.nudt, axis, cl, p + P * q, a, b, u);
                     sa[r0 + P * q] = a;
                     sb[r0 + P * q] = b;
                     su[r0 + P * q] = u;
@@ -1230,9 +1238,9 @@ __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((lon
 // precision mode, whose coefficient tables feed FP32 arithmetic only (the
 // stencil, the drift and the line-solve factors, formed from FP32-accurate
 // rows); the payoff tables stay FP64.
-template <int N, bool F32ROOT = false>
+template <int N, bool F32ROOT = false, int ST = 1, typename TC = double>
 __device__ void build_tables(const Shape<N>& s, const InstDev& P, double* tabd, double* pay,
-                             Consts<double>* cd, int rank, int gsize)
+                             TC* cst, int rank, int gsize)
 {
     const double beta = P.beta;
     const bool half = beta == 0.5;  // F^beta by a square root (the usual SABR choice)
@@ -1244,7 +1252,7 @@ __device__ void build_tables(const Shape<N>& s, const InstDev& P, double* tabd, 
         if (w >= nrate) {
             const int jj = w - nrate + 1;
             const double V = (double)jj * (P.Fmax[N - 1] * pow2(-s.lv[N - 1]));  // h_V = Vmax / M_V exactly
-            tabd[s.toff[N - 1] + jj - 1] = V * V;
+            tabd[(s.toff[N - 1] + jj - 1) * ST] = V * V;
             continue;
         }
         int a = 0, jj = w;
@@ -1257,15 +1265,15 @@ __device__ void build_tables(const Shape<N>& s, const InstDev& P, double* tabd, 
         const double al = P.alpha[a], ta = P.tau[a];
         const double F = (double)jj * h;
         const double bF = 1.0 / (1.0 + ta * F);  // discount factor of the accrual period
-        pay[s.poff[a] + jj] = (P.payoff == 0) ? (F - P.K) : ta * (F - P.K);
-        pay[s.phalf + s.poff[a] + jj] = bF;
+        pay[(s.poff[a] + jj) * ST] = (P.payoff == 0) ? (F - P.K) : ta * (F - P.K);
+        pay[(s.phalf + s.poff[a] + jj) * ST] = bF;
         if (jj >= 1) {
             const double dcoef = P.dcb[a] * pow2(2 * s.lv[a]);  // alpha^2 rho_aa / (2 h^2)
             const double Fb = half ? (F32ROOT ? (double)sqrtf((float)F) : sqrt(F)) : pow(F, beta);
             const double F2b = half ? F : pow(F, 2.0 * beta);
-            tabd[s.toff[a] + jj - 1] = dcoef * F2b;
-            tabd[s.toff[a] + M + jj - 1] = al * Fb;
-            tabd[s.toff[a] + 2 * M + jj - 1] = al * ta * Fb * bF;
+            tabd[(s.toff[a] + jj - 1) * ST] = dcoef * F2b;
+            tabd[(s.toff[a] + M + jj - 1) * ST] = al * Fb;
+            tabd[(s.toff[a] + 2 * M + jj - 1) * ST] = al * ta * Fb * bF;
         }
     }
     // the constants, one entry per lane at a time
@@ -1273,10 +1281,10 @@ __device__ void build_tables(const Shape<N>& s, const InstDev& P, double* tabd, 
     constexpr int kConsts = 1 + kPairs + kTri + 2 * kMaxDim;
     for (int q = rank; q < kConsts; q += gsize) {
         if (q == 0) {
-            cd->cV = P.cVb * pow2(2 * s.lv[N - 1]);  // sigma^2 / (2 h_V^2)
-            cd->dt = P.dt;
-            cd->thdt = P.theta * P.dt;
-            cd->nudt = P.nu * P.dt;
+            cst[0 * ST] = (TC)(P.cVb * pow2(2 * s.lv[N - 1]));  // sigma^2 / (2 h_V^2)
+            cst[1 * ST] = (TC)P.dt;
+            cst[2 * ST] = (TC)(P.theta * P.dt);
+            cst[3 * ST] = (TC)(P.nu * P.dt);
         } else if (q <= kPairs) {  // rm[upair(i, k)] = rho_ik / (4 h_i h_k), i < k
             int i = 0, r = q - 1;
             while (r >= kMaxDim - 1 - i) {
@@ -1285,20 +1293,20 @@ __device__ void build_tables(const Shape<N>& s, const InstDev& P, double* tabd, 
             }
             const int k = i + 1 + r;
             const bool ok = i < N - 1 && k < N - 1;
-            cd->rm[upair(i, k)] = ok ? P.rmb[upair(i, k)] * pow2(s.lv[i] + s.lv[k]) : 0.0;
+            cst[(kOffRm + upair(i, k)) * ST] = (TC)(ok ? P.rmb[upair(i, k)] * pow2(s.lv[i] + s.lv[k]) : 0.0);
         } else if (q <= kPairs + kTri) {  // rh[ltri(i, r)], r <= i
             int i = 0, r = q - 1 - kPairs;
             while (r > i) {
                 r -= i + 1;
                 ++i;
             }
-            cd->rh[ltri(i, r)] = (i < N - 1) ? P.rho[i * kMaxDim + r] : 0.0;
+            cst[(kOffRh + ltri(i, r)) * ST] = (TC)((i < N - 1) ? P.rho[i * kMaxDim + r] : 0.0);
         } else if (q <= kPairs + kTri + kMaxDim) {  // sigma phi_i / (4 h_i h_V)
             const int i = q - 1 - kPairs - kTri;
-            cd->sm[i] = (i < N - 1) ? P.smb[i] * pow2(s.lv[i] + s.lv[N - 1]) : 0.0;
+            cst[(kOffSm + i) * ST] = (TC)((i < N - 1) ? P.smb[i] * pow2(s.lv[i] + s.lv[N - 1]) : 0.0);
         } else {  // 1 / (2 h_i)
             const int i = q - 1 - kPairs - kTri - kMaxDim;
-            cd->g2[i] = (i < N) ? P.g2b[i] * pow2(s.lv[i]) : 0.0;
+            cst[(kOffG2 + i) * ST] = (TC)((i < N) ? P.g2b[i] * pow2(s.lv[i]) : 0.0);
         }
     }
 }
@@ -1511,7 +1519,7 @@ __device__ void solve_item(const SolveArgs& a, const Item& it, unsigned char* ba
     const int Lp = lay.Lp;
 
     // 1. coefficient and payoff tables, constants
-    build_tables<N>(s, P, tabd, pay, cd, rank, gsize);
+    build_tables<N>(s, P, tabd, pay, (double*)cd, rank, gsize);
     gsync<WARP>(gm);
     if constexpr (MIXED) {
         for (int q = rank; q < lay.ntab; q += gsize) tabk[q] = (TK)tabd[q];
@@ -1531,8 +1539,8 @@ __device__ void solve_item(const SolveArgs& a, const Item& it, unsigned char* ba
         decode<N>(s, tr, j);
         if (dirichlet_node(s, tr)) H[tr] = TK(0);
         else if constexpr (MIXED) H[tr] = (TK)payoff_H_fast<N>(s, pay, P.payoff, j, (const float*)tabk,
-                                                               *(const Consts<float>*)ck);
-        else H[tr] = (TK)payoff_H<N>(s, pay, P.payoff, j, tabd, *cd);
+                                                               (const float*)ck);
+        else H[tr] = (TK)payoff_H<N>(s, pay, P.payoff, j, tabd, (const double*)cd);
     }
     for (int t = rank; t < s.L; t += gsize) {
         const int J = s.padded(t);
@@ -1927,18 +1935,18 @@ __device__ void solve_item_mixed(const SolveArgs& a, const Item& it, unsigned ch
     float* Kw = reinterpret_cast<float*>(base + lay.Kw);
 
     // 1. coefficient and payoff tables, constants, line-solve factors
-    build_tables<N, true>(s, P, tabd, pay, cd, rank, gsize);
+    build_tables<N, true>(s, P, tabd, pay, (double*)cd, rank, gsize);
     gsync<WARP>(gm);
     for (int q = rank; q < lay.ntab; q += gsize) tabk[q] = (float)tabd[q];
     convert_consts<float>(*cd, ck, rank, gsize);
     pcr_setup<N, float, RMAX, float>(s, tabd, *cd, lu, rank, gsize, gm);
-    dense_setup<N>(s, tabd, *cd, lu, rank, gsize);
+    dense_setup<N>(s, tabd, cd->cV, cd->nudt, lu, rank, gsize);
     gsync<WARP>(gm);  // the FP32 tables and constants are complete
     // 2. H = F(G)/V^2 on the rate grid (payoff differences in FP64), Z from the state or zero
     for (int tr = rank; tr < s.Lr; tr += gsize) {
         int j[N];
         decode<N>(s, tr, j);
-        H[tr] = dirichlet_node(s, tr) ? 0.f : payoff_H_fast<N>(s, pay, P.payoff, j, tabk, *ck);
+        H[tr] = dirichlet_node(s, tr) ? 0.f : payoff_H_fast<N>(s, pay, P.payoff, j, tabk, (const float*)ck);
     }
     for (int t = rank; t < s.L; t += gsize) {
         const int J = s.padded(t);
@@ -2166,66 +2174,4 @@ __global__ void __launch_bounds__(KIND == kWarpGroup ? 128 : kCtaMaxThreads, KIN
     }
 }
 
-// Host launch / occupancy helpers, instantiated once per N.
-template <int N>
-const void* kernel_for(bool mixed, int kind)
-{
-    if (kind == kWarpGroup)
-        return mixed ? (const void*)solve_kernel<N, true, kWarpGroup> : (const void*)solve_kernel<N, false, kWarpGroup>;
-    if (kind == kCtaGroup)
-        return mixed ? (const void*)solve_kernel<N, true, kCtaGroup> : (const void*)solve_kernel<N, false, kCtaGroup>;
-    return mixed ? (const void*)solve_kernel<N, true, kMemGroup> : (const void*)solve_kernel<N, false, kMemGroup>;
-}
-
-template <int N>
-int launch_impl(const SolveArgs& a, bool mixed, int kind, int block, int grid, size_t smem, void* stream)
-{
-    cudaStream_t st = (cudaStream_t)stream;
-    if (kind == kWarpGroup) {
-        if (mixed) solve_kernel<N, true, kWarpGroup><<<grid, block, smem, st>>>(a);
-        else solve_kernel<N, false, kWarpGroup><<<grid, block, smem, st>>>(a);
-    } else if (kind == kCtaGroup) {
-        if (mixed) solve_kernel<N, true, kCtaGroup><<<grid, block, smem, st>>>(a);
-        else solve_kernel<N, false, kCtaGroup><<<grid, block, smem, st>>>(a);
-    } else {
-        if (mixed) solve_kernel<N, true, kMemGroup><<<grid, block, smem, st>>>(a);
-        else solve_kernel<N, false, kMemGroup><<<grid, block, smem, st>>>(a);
-    }
-    return (int)cudaGetLastError();
-}
-
-template <int N>
-int occupancy_impl(bool mixed, int kind, int block, size_t smem)
-{
-    int nb = 0;
-    const void* f = kernel_for<N>(mixed, kind);
-    // The limit is an attribute of the kernel, shared by all its launches, and
-    // launches of one kernel request different amounts: past the default
-    // 48 KB, allow the device's opt-in maximum (less the kernel's static
-    // shared memory), so that no launch depends on which query came last.
-    if (smem > 48 * 1024) {
-        int dev = 0, optin = 0;
-        cudaFuncAttributes fa{};
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-            cudaFuncGetAttributes(&fa, f) != cudaSuccess)
-            return 0;
-        const int lim = optin - (int)fa.sharedSizeBytes;
-        if ((size_t)lim < smem ||
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess)
-            return 0;
-    }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem) != cudaSuccess) return 0;
-    return nb;
-}
-
 }  // namespace amfrw
-
-#define AMFRW_INSTANTIATE(NN)                                                               \
-    namespace amfrw {                                                                       \
-    int launch_n##NN(const SolveArgs& a, bool m, int k, int b, int g, size_t s, void* st)   \
-    {                                                                                       \
-        return launch_impl<NN>(a, m, k, b, g, s, st);                                       \
-    }                                                                                       \
-    int occupancy_n##NN(bool m, int k, int b, size_t s) { return occupancy_impl<NN>(m, k, b, s); } \
-    }
