@@ -77,14 +77,14 @@ int gemm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M
     // (A's tiles come from L2).
     int BN = N <= 256 ? N : 256;
     const int rt = (M + kBM - 1) / kBM, sms = device_sms(dev);
-    while (BN % 32 == 0 && BN > 32 && rt * ((N + BN - 1) / BN) * 2 <= sms) BN /= 2;
+    while (epi.mode != 3 && BN % 32 == 0 && BN > 32 && rt * ((N + BN - 1) / BN) * 2 <= sms) BN /= 2;
     const int nk = (K + kBK - 1) / kBK;
     // at most two stages of the widest tile (96 KB), so that two CTAs share an
     // SM and one's epilogue overlaps the other's loads and MMAs
     int S = kMaxStages;
     while (S > 1 && (S > nk || smem_bytes(BN, S) > 112 * 1024)) --S;
-    // (the epilogue turns 4 x 4.5 KB through the stages' memory)
-    const int smem = std::max(smem_bytes(BN, S), 1024 + 4 * 32 * 144);
+    // (the epilogue turns its values through the stages' memory)
+    const int smem = std::max(smem_bytes(BN, S), 1024 + kThreads / 32 * kTurnBytes);
     // The dynamic shared-memory limit is a per-device attribute of the
     // kernel: raise it once on every device that launches it (to the most any
     // launch asks for).
@@ -188,6 +188,7 @@ constexpr int ob3 = oW3 + kW * kW;
 constexpr int ow4 = ob3 + kW;
 constexpr int ob4 = ow4 + kW;
 constexpr int kParams = ob4 + 1;
+static_assert(ob4 == ow4 + kW, "the output product reads b4 behind w4");
 // control variate: every monomial of degree <= 3 in the 8 normalised features
 constexpr int kPolyTerms = 1 + kIn + kIn * (kIn + 1) / 2 + kIn * (kIn + 1) * (kIn + 2) / 6;
 
@@ -215,21 +216,101 @@ inline void poly_terms(const float* z, double* m)
     poly_each(z, [m](int q, double v) { m[q] = v; });
 }
 
-// g_b = poly(z_b) + ymu + ysd * mean_b: the predicted target (log price or
-// price) in FP64, from the ensemble mean of the standardised residual.
-__global__ void finish_kernel(const float* __restrict__ z, const double* __restrict__ coef,
-                              const float* __restrict__ mean, int n, double ymu, double ysd, double* g)
+// The feature box: a surrogate's normalisation and lattices.
+struct Box {
+    double fmin[kIn], fmax[kIn];
+    int nlat[kIn];
+    double lat[kIn][kMaxLattice];
+};
+
+// Feature c of a row normalised to [-1, 1] over the box; `ok` is cleared
+// outside it (and off the training values of a lattice feature).
+__host__ __device__ inline float norm_feature(const Box& b, int c, double f, bool& ok)
+{
+    const double span = b.fmax[c] - b.fmin[c];
+    const double z = span > 0 ? 2.0 * (f - b.fmin[c]) / span - 1.0 : (f == b.fmin[c] ? 0.0 : 2.0);
+    if (!(z >= -1.0 - 1e-9 && z <= 1.0 + 1e-9)) ok = false;
+    if (b.nlat[c] > 0) {  // a lattice feature: only its training values
+        const double tol = 1e-12 * fmax(1.0, fabs(f));
+        bool on = false;
+        for (int q = 0; q < b.nlat[c] && !on; ++q) on = fabs(f - b.lat[c][q]) <= tol;
+        if (!on) ok = false;
+    }
+    return (float)z;
+}
+
+// Query rows (raw features, FP64): normalised features z [n x 8], the
+// network's BF16 input X [n x 16] (8 zeros behind them) and whether the row
+// lies in the box.  A thread per feature; the row's eight threads agree on ok.
+__global__ void __launch_bounds__(256) query_kernel(const double* __restrict__ raw, int n, const Box* __restrict__ box,
+                                                    float* z, bf16* X, uint8_t* ok)
+{
+    __shared__ Box b;
+    for (int q = threadIdx.x; q < (int)(sizeof(Box) / 4); q += blockDim.x)
+        reinterpret_cast<int*>(&b)[q] = reinterpret_cast<const int*>(box)[q];
+    __syncthreads();
+    const int q = blockIdx.x * blockDim.x + threadIdx.x, r = q / kIn, c = q % kIn;
+    bool in = true;
+    float v = 0.0f;
+    if (r < n) v = norm_feature(b, c, raw[q], in);
+    for (int o = 1; o < kIn; o <<= 1) in = __shfl_xor_sync(0xffffffffu, (int)in, o) && in;
+    if (r >= n) return;
+    z[q] = v;
+    X[(size_t)r * kInPad + c] = __float2bfloat16(v);
+    X[(size_t)r * kInPad + kIn + c] = __float2bfloat16(0.0f);
+    if (c == 0) ok[r] = in ? 1 : 0;
+}
+
+// Predictions of n rows from the members' outputs ys [members x n]: the
+// ensemble's mean and sample standard deviation, g = poly(z) + ymu + ysd mean
+// (the target: log price or price) and from it the price and its spread to
+// first order, in FP64.  The cubic is nested by feature (164 multiply-adds a
+// row; forming the monomials one by one took 74 us for 65536 rows, this 31).
+__global__ void __launch_bounds__(128) finish_kernel(const float* __restrict__ z, const double* __restrict__ coef,
+                                                     const float* __restrict__ ys, int members, int n, double ymu,
+                                                     double ysd, int log_target, double* mean_out, double* spread_out)
 {
     __shared__ double c[kPolyTerms];
     for (int q = threadIdx.x; q < kPolyTerms; q += blockDim.x) c[q] = coef[q];
     __syncthreads();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= n) return;
-    float zb[kIn];
-    for (int i = 0; i < kIn; ++i) zb[i] = z[(size_t)b * kIn + i];
-    double acc = 0.0;
-    poly_each(zb, [&](int q, double v) { acc += c[q] * v; });
-    g[b] = acc + ymu + ysd * (double)mean[b];
+    float s = 0.0f;
+    for (int m = 0; m < members; ++m) s += ys[(size_t)m * n + b];
+    const float mu = s / (float)members;
+    float v = 0.0f;
+    for (int m = 0; m < members; ++m) {
+        const float d = ys[(size_t)m * n + b] - mu;
+        v += d * d;
+    }
+    const float sd = members > 1 ? sqrtf(v / (float)(members - 1)) : 0.0f;
+    double x[kIn];
+#pragma unroll
+    for (int i = 0; i < kIn; ++i) x[i] = (double)z[(size_t)b * kIn + i];
+    // 1, z_i, z_i z_j (i <= j), z_i z_j z_k (i <= j <= k), in poly_each's order
+    double acc = c[0];
+    int q2 = 1 + kIn, q3 = 1 + kIn + kIn * (kIn + 1) / 2;
+#pragma unroll
+    for (int i = 0; i < kIn; ++i) {
+        double li = c[1 + i];
+#pragma unroll
+        for (int j = i; j < kIn; ++j) {
+            double qij = c[q2++];
+#pragma unroll
+            for (int k = j; k < kIn; ++k) qij = fma(c[q3++], x[k], qij);
+            li = fma(qij, x[j], li);
+        }
+        acc = fma(li, x[i], acc);
+    }
+    const double g = acc + ymu + ysd * (double)mu, sp = ysd * (double)sd;
+    if (log_target) {
+        const double p = exp(g);
+        mean_out[b] = p;
+        spread_out[b] = p * sp;
+    } else {
+        mean_out[b] = g;
+        spread_out[b] = sp;
+    }
 }
 
 // Batch of rows (gathered through idx, or consecutive from r0) as BF16 input
@@ -354,23 +435,6 @@ __global__ void cast_kernel(const float* __restrict__ W, int rows, int cols, bf1
     const bf16 h = __float2bfloat16(W[i]);
     Wb[i] = h;
     if (Wtb) Wtb[(size_t)c * rows + r] = h;
-}
-
-// Ensemble mean and sample standard deviation of the members' outputs.
-__global__ void ensemble_kernel(const float* __restrict__ ys, int members, int n, float* mean, float* spread)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.0f;
-    for (int m = 0; m < members; ++m) s += ys[(size_t)m * n + i];
-    const float mu = s / (float)members;
-    float q = 0.0f;
-    for (int m = 0; m < members; ++m) {
-        const float d = ys[(size_t)m * n + i] - mu;
-        q += d * d;
-    }
-    mean[i] = mu;
-    spread[i] = members > 1 ? sqrtf(q / (float)(members - 1)) : 0.0f;
 }
 
 inline int cdiv(int a, int b) { return (a + b - 1) / b; }
@@ -543,16 +607,19 @@ struct amfrw_surrogate {
     std::vector<bf16*> W1b, W2b, W3b, W2tb, W3tb;
     SgWork w;                  // prediction chunk (kPredRows) and gradient checks (kTrainRows)
     float* ys = nullptr;       // prediction chunk: every member's output
-    float *pmean = nullptr, *pspread = nullptr;  // prediction chunk: ensemble mean, spread
-    double *pg = nullptr, *dpoly = nullptr;      // prediction chunk: target; control-variate coefficients
+    // prediction chunk: raw and normalised features, prices, spreads, in-box flags
+    double *praw = nullptr, *pmean = nullptr, *pspread = nullptr;
+    float* pz = nullptr;
+    uint8_t* pok = nullptr;
+    double* dpoly = nullptr;   // control-variate coefficients
+    Box* dbox = nullptr;
     int* err = nullptr;
     double poly[kPolyTerms] = {};
     int adam_t = 0;
-    double fmin[kIn], fmax[kIn];
-    // features that took at most kMaxLattice distinct values in the training
-    // set (a lattice, e.g. strikes): queries must lie on one of them
-    int nlat[kIn] = {};
-    double lat[kIn][kMaxLattice] = {};
+    // the box: fmin, fmax; features that took at most kMaxLattice distinct
+    // values in the training set (a lattice, e.g. strikes): queries must lie
+    // on one of them
+    Box box{};
     double ymu = 0.0, ysd = 1.0;    // target scaling: t = (g(price) - ymu) / ysd
     bool log_target = false;        // g = log (all training prices > 0), else identity
     double calib = 0.0, rel_bound = 1e-3;
@@ -565,7 +632,9 @@ struct amfrw_surrogate {
         for (auto v : {&W1b, &W2b, &W3b, &W2tb, &W3tb})
             for (bf16* q : *v) cudaFree(q);
         w.release();
-        for (void* q : {(void*)ys, (void*)err, (void*)pmean, (void*)pspread, (void*)pg, (void*)dpoly}) cudaFree(q);
+        for (void* q : {(void*)ys, (void*)err, (void*)praw, (void*)pz, (void*)pok, (void*)pmean, (void*)pspread, (void*)dpoly,
+                        (void*)dbox})
+            cudaFree(q);
     }
 };
 
@@ -614,9 +683,12 @@ int sg_alloc(amfrw_surrogate* s)
     if (st != AMFRW_OK) return st;
     SG_CUDA(cudaMalloc(&s->ys, F4 * PQ * (size_t)s->members));
     SG_CUDA(cudaMalloc(&s->err, sizeof(int)));
-    SG_CUDA(cudaMalloc(&s->pmean, F4 * PR));
-    SG_CUDA(cudaMalloc(&s->pspread, F4 * PR));
-    SG_CUDA(cudaMalloc(&s->pg, sizeof(double) * PR));
+    SG_CUDA(cudaMalloc(&s->praw, sizeof(double) * PR * kIn));
+    SG_CUDA(cudaMalloc(&s->pz, F4 * PR * kIn));
+    SG_CUDA(cudaMalloc(&s->pok, PR));
+    SG_CUDA(cudaMalloc(&s->pmean, sizeof(double) * PR));
+    SG_CUDA(cudaMalloc(&s->pspread, sizeof(double) * PR));
+    SG_CUDA(cudaMalloc(&s->dbox, sizeof(Box)));
     SG_CUDA(cudaMalloc(&s->dpoly, sizeof(double) * kPolyTerms));
     SG_CUDA(cudaMemsetAsync(s->dpoly, 0, sizeof(double) * kPolyTerms, s->stream));
     SG_CUDA(cudaMemsetAsync(s->err, 0, sizeof(int), s->stream));
@@ -645,8 +717,13 @@ int sg_forward(amfrw_surrogate* s, int m, int B, bool train, float* y, const SgW
     e.bias = s->P[m] + ob2; e.Z = train ? w.Z2 : nullptr; e.H = w.H2; e.Ht = train ? w.H2t : nullptr;
     if (!rc) rc = tc::gemm(w.H1, kW, s->W2b[m], kW, B, kW, kW, e, st);
     e.bias = s->P[m] + ob3; e.Z = train ? w.Z3 : nullptr; e.H = w.H3; e.Ht = nullptr;
+    // a prediction needs the third layer's activations only in its output,
+    // which the product's epilogue forms (out_fwd_kernel's sum in its order)
+    e.mode = train ? 1 : 3;
+    e.w4 = s->P[m] + ow4;
+    e.y = y;
     if (!rc) rc = tc::gemm(w.H2, kW, s->W3b[m], kW, B, kW, kW, e, st);
-    if (!rc) out_fwd_kernel<<<cdiv(B * 32, 256), 256, 0, st>>>(w.H3, s->P[m], y, B);
+    if (!rc && train) out_fwd_kernel<<<cdiv(B * 32, 256), 256, 0, st>>>(w.H3, s->P[m], y, B);
     if (rc) return sg_fail(AMFRW_ECUDA, std::string("surrogate forward: ") + cudaGetErrorString((cudaError_t)rc));
     return AMFRW_OK;
 }
@@ -743,26 +820,13 @@ bool fit_poly(const float* z, const double* g, int64_t n, double* coef)
     return true;
 }
 
-// Normalised features (host, n x 8 floats) of n rows of raw features; ok
-// entries (may be NULL) cleared for rows outside the trained feature box.
-void sg_normalise(const amfrw_surrogate* s, const double* raw, int64_t n, std::vector<float>& out, char* ok)
+// Normalised features (host, n x 8 floats) of n training rows of raw features.
+void sg_normalise(const amfrw_surrogate* s, const double* raw, int64_t n, std::vector<float>& out)
 {
     out.assign((size_t)n * kIn, 0.0f);
-    for (int64_t i = 0; i < n; ++i) {
-        for (int c = 0; c < kIn; ++c) {
-            const double f = raw[(size_t)i * kIn + c];
-            const double span = s->fmax[c] - s->fmin[c];
-            const double z = span > 0 ? 2.0 * (f - s->fmin[c]) / span - 1.0 : (f == s->fmin[c] ? 0.0 : 2.0);
-            if (ok && !(z >= -1.0 - 1e-9 && z <= 1.0 + 1e-9)) ok[i] = 0;
-            if (ok && s->nlat[c] > 0) {  // a lattice feature: only its training values
-                bool on = false;
-                for (int q = 0; q < s->nlat[c] && !on; ++q)
-                    on = std::fabs(f - s->lat[c][q]) <= 1e-12 * std::max(1.0, std::fabs(f));
-                if (!on) ok[i] = 0;
-            }
-            out[(size_t)i * kIn + c] = (float)z;
-        }
-    }
+    bool ok = true;
+    for (int64_t i = 0; i < n; ++i)
+        for (int c = 0; c < kIn; ++c) out[(size_t)i * kIn + c] = norm_feature(s->box, c, raw[(size_t)i * kIn + c], ok);
 }
 
 // Raw features of n instances and whether each belongs to the family.
@@ -777,66 +841,47 @@ void sg_raw_features(const amfrw_surrogate* s, const amfrw_params* ps, int64_t n
     }
 }
 
-// Ensemble mean and spread (price units) of n rows of normalised features on
-// the device.
-int sg_predict_dev(amfrw_surrogate* s, const float* d_feats, int64_t n, std::vector<double>& mean,
-                   std::vector<double>& spread)
+// Prices, spreads (price units) and in-box flags of n rows of raw features, all
+// host arrays, in chunks of kPredRows.
+int sg_predict_raw(amfrw_surrogate* s, const double* raw, int64_t n, double* mean, double* spread, uint8_t* ok)
 {
     cudaStream_t st = s->stream;
-    mean.assign((size_t)n, 0.0);
-    spread.assign((size_t)n, 0.0);
-    std::vector<double> hg;
-    std::vector<float> hs;
     for (int64_t r0 = 0; r0 < n; r0 += kPredRows) {
         const int B = (int)std::min<int64_t>(kPredRows, n - r0);
-        const float* z = d_feats + (size_t)r0 * kIn;
-        pack_kernel<<<cdiv(B * kInPad, 256), 256, 0, st>>>(z, nullptr, nullptr, 0, B, s->w.X, nullptr, nullptr);
+        SG_CUDA(cudaMemcpyAsync(s->praw, raw + (size_t)r0 * kIn, sizeof(double) * B * kIn, cudaMemcpyHostToDevice, st));
+        query_kernel<<<cdiv(B * kIn, 256), 256, 0, st>>>(s->praw, B, s->dbox, s->pz, s->w.X, s->pok);
         for (int m = 0; m < s->members; ++m) {
             const int rc = sg_forward(s, m, B, false, s->ys + (size_t)m * B, s->w);
             if (rc != AMFRW_OK) return rc;
         }
-        ensemble_kernel<<<cdiv(B, 256), 256, 0, st>>>(s->ys, s->members, B, s->pmean, s->pspread);
-        finish_kernel<<<cdiv(B, 128), 128, 0, st>>>(z, s->dpoly, s->pmean, B, s->ymu, s->ysd, s->pg);
-        hg.resize(B);
-        hs.resize(B);
-        SG_CUDA(cudaMemcpyAsync(hg.data(), s->pg, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
-        SG_CUDA(cudaMemcpyAsync(hs.data(), s->pspread, sizeof(float) * B, cudaMemcpyDeviceToHost, st));
-        SG_CUDA(cudaStreamSynchronize(st));
-        for (int i = 0; i < B; ++i) {
-            const double g = hg[i], sp = s->ysd * (double)hs[i];
-            if (s->log_target) {  // spread to first order in price units
-                mean[(size_t)(r0 + i)] = std::exp(g);
-                spread[(size_t)(r0 + i)] = std::exp(g) * sp;
-            } else {
-                mean[(size_t)(r0 + i)] = g;
-                spread[(size_t)(r0 + i)] = sp;
-            }
-        }
+        finish_kernel<<<cdiv(B, 128), 128, 0, st>>>(s->pz, s->dpoly, s->ys, s->members, B, s->ymu, s->ysd,
+                                                    s->log_target ? 1 : 0, s->pmean, s->pspread);
+        SG_CUDA(cudaMemcpyAsync(mean + r0, s->pmean, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
+        SG_CUDA(cudaMemcpyAsync(spread + r0, s->pspread, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
+        SG_CUDA(cudaMemcpyAsync(ok + r0, s->pok, B, cudaMemcpyDeviceToHost, st));
     }
     return sg_check_err(s);
 }
 
-// Prediction from raw features; ok (n entries, set by the caller for family
-// membership) is cleared where a row leaves the feature box.
-int sg_predict_raw(amfrw_surrogate* s, const double* raw, int64_t n, std::vector<double>& mean,
-                   std::vector<double>& spread, std::vector<char>& ok)
-{
-    std::vector<float> feats;
-    sg_normalise(s, raw, n, feats, ok.data());
-    float* d = nullptr;
-    SG_CUDA(cudaMalloc(&d, sizeof(float) * std::max<size_t>(1, feats.size())));
-    cudaMemcpyAsync(d, feats.data(), sizeof(float) * feats.size(), cudaMemcpyHostToDevice, s->stream);
-    const int st = sg_predict_dev(s, d, n, mean, spread);
-    cudaFree(d);
-    return st;
-}
-
-int sg_predict_host(amfrw_surrogate* s, const amfrw_params* ps, int64_t n, std::vector<double>& mean,
-                    std::vector<double>& spread, std::vector<char>& ok)
+// The same for instances; ok is also cleared outside the family.
+int sg_predict_host(amfrw_surrogate* s, const amfrw_params* ps, int64_t n, double* mean, double* spread, uint8_t* ok)
 {
     std::vector<double> raw;
-    sg_raw_features(s, ps, n, raw, ok);
-    return sg_predict_raw(s, raw.data(), n, mean, spread, ok);
+    std::vector<char> fam;
+    sg_raw_features(s, ps, n, raw, fam);
+    const int st = sg_predict_raw(s, raw.data(), n, mean, spread, ok);
+    if (st != AMFRW_OK) return st;
+    for (int64_t i = 0; i < n; ++i) ok[i] = ok[i] && fam[(size_t)i] ? 1 : 0;
+    return AMFRW_OK;
+}
+
+void sg_copy_out(int64_t n, const std::vector<double>& mean, const std::vector<double>& spread,
+                 const std::vector<uint8_t>& ok, double* mean_out, double* spread_out, uint8_t* ok_out)
+{
+    if (n < 1) return;
+    memcpy(mean_out, mean.data(), sizeof(double) * (size_t)n);
+    memcpy(spread_out, spread.data(), sizeof(double) * (size_t)n);
+    if (ok_out) memcpy(ok_out, ok.data(), (size_t)n);
 }
 
 // Answers from the network where the calibrated estimate is within the bound;
@@ -844,7 +889,7 @@ int sg_predict_host(amfrw_surrogate* s, const amfrw_params* ps, int64_t n, std::
 // most 4096 instances each).  param(i) gives query i as amfrw_params.
 template <class ParamOf>
 int sg_serve(amfrw_surrogate* s, int64_t n, const std::vector<double>& mean, const std::vector<double>& spread,
-             const std::vector<char>& ok, ParamOf param, double* prices_out, uint8_t* fell_back_out,
+             const std::vector<uint8_t>& ok, ParamOf param, double* prices_out, uint8_t* fell_back_out,
              void* cuda_stream)
 {
     std::vector<int64_t> where;
@@ -934,8 +979,8 @@ int amfrw_surrogate_fit(amfrw_surrogate* s, const amfrw_params* ps, const double
     // family, feature box and target scaling from the training set
     s->fam = family_of(ps[0]);
     for (int c = 0; c < kIn; ++c) {
-        s->fmin[c] = 1e300;
-        s->fmax[c] = -1e300;
+        s->box.fmin[c] = 1e300;
+        s->box.fmax[c] = -1e300;
     }
     std::vector<double> raw;
     std::vector<char> ok;
@@ -946,15 +991,15 @@ int amfrw_surrogate_fit(amfrw_surrogate* s, const amfrw_params* ps, const double
         if (!std::isfinite(prices[i])) return sg_fail(AMFRW_EINVAL, "non-finite training price");
         positive = positive && prices[i] > 0.0;
         for (int c = 0; c < kIn; ++c) {
-            s->fmin[c] = std::min(s->fmin[c], raw[(size_t)i * kIn + c]);
-            s->fmax[c] = std::max(s->fmax[c], raw[(size_t)i * kIn + c]);
+            s->box.fmin[c] = std::min(s->box.fmin[c], raw[(size_t)i * kIn + c]);
+            s->box.fmax[c] = std::max(s->box.fmax[c], raw[(size_t)i * kIn + c]);
         }
     }
     // features with at most kMaxLattice distinct training values (and more
     // than one) are lattices: the network is trained, and answers, only there
     for (int c = 0; c < kIn; ++c) {
         std::vector<double> v;
-        s->nlat[c] = 0;
+        s->box.nlat[c] = 0;
         for (int64_t i = 0; i < n && (int)v.size() <= kMaxLattice; ++i) {
             const double x = raw[(size_t)i * kIn + c];
             bool seen = false;
@@ -963,8 +1008,8 @@ int amfrw_surrogate_fit(amfrw_surrogate* s, const amfrw_params* ps, const double
         }
         if (v.size() >= 2 && (int)v.size() <= kMaxLattice) {
             std::sort(v.begin(), v.end());
-            s->nlat[c] = (int)v.size();
-            for (size_t q = 0; q < v.size(); ++q) s->lat[c][q] = v[q];
+            s->box.nlat[c] = (int)v.size();
+            for (size_t q = 0; q < v.size(); ++q) s->box.lat[c][q] = v[q];
         }
     }
     // the network learns log(price) when every price is positive (its squared
@@ -973,7 +1018,7 @@ int amfrw_surrogate_fit(amfrw_surrogate* s, const amfrw_params* ps, const double
     std::vector<double> g((size_t)n);
     for (int64_t i = 0; i < n; ++i) g[(size_t)i] = positive ? std::log(prices[i]) : prices[i];
     std::vector<float> feats, targ((size_t)n);
-    sg_normalise(s, raw.data(), n, feats, nullptr);
+    sg_normalise(s, raw.data(), n, feats);
     // control variate: least-squares cubic in the features; the networks
     // learn what it leaves, standardised
     if (!fit_poly(feats.data(), g.data(), n, s->poly)) return sg_fail(AMFRW_EINVAL, "control-variate fit failed");
@@ -990,6 +1035,7 @@ int amfrw_surrogate_fit(amfrw_surrogate* s, const amfrw_params* ps, const double
     s->ysd = std::sqrt(std::max(sq / (double)n - s->ymu * s->ymu, 1e-300));
     for (int64_t i = 0; i < n; ++i) targ[(size_t)i] = (float)((g[(size_t)i] - s->ymu) / s->ysd);
     SG_CUDA(cudaMemcpyAsync(s->dpoly, s->poly, sizeof(double) * kPolyTerms, cudaMemcpyHostToDevice, s->stream));
+    SG_CUDA(cudaMemcpyAsync(s->dbox, &s->box, sizeof(Box), cudaMemcpyHostToDevice, s->stream));
     cudaStream_t st = s->stream;
     float *d_feats = nullptr, *d_targ = nullptr;
     SG_CUDA(cudaMalloc(&d_feats, sizeof(float) * feats.size()));
@@ -1090,15 +1136,12 @@ int amfrw_surrogate_predict(amfrw_surrogate* s, const amfrw_params* ps, int64_t 
 {
     if (!s || !ps || !mean_out || !spread_out) return sg_fail(AMFRW_EINVAL, "NULL argument");
     if (!s->trained) return sg_fail(AMFRW_EINVAL, "surrogate is not trained");
-    std::vector<double> mean, spread;
-    std::vector<char> ok;
-    int st = sg_predict_host(s, ps, n, mean, spread, ok);
+    // (nothing is written on error)
+    std::vector<double> mean((size_t)std::max<int64_t>(n, 0)), spread(mean.size());
+    std::vector<uint8_t> ok(mean.size());
+    const int st = sg_predict_host(s, ps, n, mean.data(), spread.data(), ok.data());
     if (st != AMFRW_OK) return st;
-    for (int64_t i = 0; i < n; ++i) {
-        mean_out[i] = mean[(size_t)i];
-        spread_out[i] = spread[(size_t)i];
-        if (in_domain_out) in_domain_out[i] = ok[(size_t)i] ? 1 : 0;
-    }
+    sg_copy_out(n, mean, spread, ok, mean_out, spread_out, in_domain_out);
     return AMFRW_OK;
 }
 
@@ -1108,15 +1151,11 @@ int amfrw_surrogate_predict_features(amfrw_surrogate* s, const double* features,
     if (!s || !features || !mean_out || !spread_out) return sg_fail(AMFRW_EINVAL, "NULL argument");
     if (n < 0) return sg_fail(AMFRW_EINVAL, "n < 0");
     if (!s->trained) return sg_fail(AMFRW_EINVAL, "surrogate is not trained");
-    std::vector<double> mean, spread;
-    std::vector<char> ok((size_t)n, 1);
-    int st = sg_predict_raw(s, features, n, mean, spread, ok);
+    std::vector<double> mean((size_t)n), spread((size_t)n);
+    std::vector<uint8_t> ok((size_t)n);
+    const int st = sg_predict_raw(s, features, n, mean.data(), spread.data(), ok.data());
     if (st != AMFRW_OK) return st;
-    for (int64_t i = 0; i < n; ++i) {
-        mean_out[i] = mean[(size_t)i];
-        spread_out[i] = spread[(size_t)i];
-        if (in_box_out) in_box_out[i] = ok[(size_t)i] ? 1 : 0;
-    }
+    sg_copy_out(n, mean, spread, ok, mean_out, spread_out, in_box_out);
     return AMFRW_OK;
 }
 
@@ -1127,9 +1166,9 @@ int amfrw_surrogate_calibrate(amfrw_surrogate* s, const amfrw_params* ps, const 
     if (!s->trained) return sg_fail(AMFRW_EINVAL, "surrogate is not trained");
     if (n < 16 || !(rel_bound > 0) || !(quantile > 0 && quantile <= 1))
         return sg_fail(AMFRW_EINVAL, "need n >= 16, rel_bound > 0, quantile in (0, 1]");
-    std::vector<double> mean, spread;
-    std::vector<char> ok;
-    int st = sg_predict_host(s, ps, n, mean, spread, ok);
+    std::vector<double> mean((size_t)std::max<int64_t>(n, 0)), spread(mean.size());
+    std::vector<uint8_t> ok(mean.size());
+    int st = sg_predict_host(s, ps, n, mean.data(), spread.data(), ok.data());
     if (st != AMFRW_OK) return st;
     std::vector<double> ratio;
     for (int64_t i = 0; i < n; ++i) {
@@ -1152,9 +1191,9 @@ int amfrw_surrogate_eval(amfrw_surrogate* s, const amfrw_params* ps, int64_t n, 
 {
     if (!s || !ps || !prices_out) return sg_fail(AMFRW_EINVAL, "NULL argument");
     if (!s->trained || !s->calibrated) return sg_fail(AMFRW_EINVAL, "surrogate is not trained and calibrated");
-    std::vector<double> mean, spread;
-    std::vector<char> ok;
-    int st = sg_predict_host(s, ps, n, mean, spread, ok);
+    std::vector<double> mean((size_t)std::max<int64_t>(n, 0)), spread(mean.size());
+    std::vector<uint8_t> ok(mean.size());
+    int st = sg_predict_host(s, ps, n, mean.data(), spread.data(), ok.data());
     if (st != AMFRW_OK) return st;
     return sg_serve(
         s, n, mean, spread, ok, [&](int64_t i, InstanceStore&) { return ps[i]; }, prices_out, fell_back_out,
@@ -1169,9 +1208,9 @@ int amfrw_surrogate_eval_features(amfrw_surrogate* s, const double* features, in
     if (!s->trained || !s->calibrated) return sg_fail(AMFRW_EINVAL, "surrogate is not trained and calibrated");
     for (int64_t i = 0; i < n * kIn; ++i)
         if (!std::isfinite(features[i])) return sg_fail(AMFRW_EINVAL, "non-finite feature");
-    std::vector<double> mean, spread;
-    std::vector<char> ok((size_t)n, 1);
-    int st = sg_predict_raw(s, features, n, mean, spread, ok);
+    std::vector<double> mean((size_t)n), spread((size_t)n);
+    std::vector<uint8_t> ok((size_t)n);
+    int st = sg_predict_raw(s, features, n, mean.data(), spread.data(), ok.data());
     if (st != AMFRW_OK) return st;
     return sg_serve(
         s, n, mean, spread, ok,
@@ -1188,16 +1227,16 @@ int amfrw_surrogate_save(const amfrw_surrogate* s, const char* path)
     std::vector<float> h(kParams);
     bool ok = fwrite(magic, 1, 8, f) == 8;
     ok = ok && fwrite(&s->members, sizeof(int), 1, f) == 1;
-    ok = ok && fwrite(s->fmin, sizeof(double), kIn, f) == (size_t)kIn;
-    ok = ok && fwrite(s->fmax, sizeof(double), kIn, f) == (size_t)kIn;
+    ok = ok && fwrite(s->box.fmin, sizeof(double), kIn, f) == (size_t)kIn;
+    ok = ok && fwrite(s->box.fmax, sizeof(double), kIn, f) == (size_t)kIn;
     const double sc[4] = {s->ymu, s->ysd, s->calib, s->rel_bound};
     ok = ok && fwrite(sc, sizeof(double), 4, f) == 4;
     const int flags[3] = {s->trained ? 1 : 0, s->calibrated ? 1 : 0, s->log_target ? 1 : 0};
     ok = ok && fwrite(flags, sizeof(int), 3, f) == 3;
     ok = ok && fwrite(&s->fam, sizeof(Family), 1, f) == 1;
     ok = ok && fwrite(s->poly, sizeof(double), kPolyTerms, f) == (size_t)kPolyTerms;
-    ok = ok && fwrite(s->nlat, sizeof(int), kIn, f) == (size_t)kIn;
-    ok = ok && fwrite(s->lat, sizeof(double), kIn * kMaxLattice, f) == (size_t)(kIn * kMaxLattice);
+    ok = ok && fwrite(s->box.nlat, sizeof(int), kIn, f) == (size_t)kIn;
+    ok = ok && fwrite(s->box.lat, sizeof(double), kIn * kMaxLattice, f) == (size_t)(kIn * kMaxLattice);
     for (int m = 0; m < s->members && ok; ++m) {
         ok = cudaMemcpy(h.data(), s->P[m], sizeof(float) * kParams, cudaMemcpyDeviceToHost) == cudaSuccess;
         ok = ok && fwrite(h.data(), sizeof(float), kParams, f) == (size_t)kParams;
@@ -1221,13 +1260,14 @@ int amfrw_surrogate_load(const char* path, void* cuda_stream, amfrw_surrogate** 
     double sc[4];
     int flags[3];
     if (ok) {
-        ok = fread(s->fmin, sizeof(double), kIn, f) == (size_t)kIn && fread(s->fmax, sizeof(double), kIn, f) == (size_t)kIn;
+        ok = fread(s->box.fmin, sizeof(double), kIn, f) == (size_t)kIn && fread(s->box.fmax, sizeof(double), kIn, f) == (size_t)kIn;
         ok = ok && fread(sc, sizeof(double), 4, f) == 4 && fread(flags, sizeof(int), 3, f) == 3;
         ok = ok && fread(&s->fam, sizeof(Family), 1, f) == 1;
         ok = ok && fread(s->poly, sizeof(double), kPolyTerms, f) == (size_t)kPolyTerms;
-        ok = ok && fread(s->nlat, sizeof(int), kIn, f) == (size_t)kIn;
-        ok = ok && fread(s->lat, sizeof(double), kIn * kMaxLattice, f) == (size_t)(kIn * kMaxLattice);
-        for (int c = 0; c < kIn && ok; ++c) ok = s->nlat[c] >= 0 && s->nlat[c] <= kMaxLattice;
+        ok = ok && fread(s->box.nlat, sizeof(int), kIn, f) == (size_t)kIn;
+        ok = ok && fread(s->box.lat, sizeof(double), kIn * kMaxLattice, f) == (size_t)(kIn * kMaxLattice);
+        for (int c = 0; c < kIn && ok; ++c) ok = s->box.nlat[c] >= 0 && s->box.nlat[c] <= kMaxLattice;
+        ok = ok && cudaMemcpy(s->dbox, &s->box, sizeof(Box), cudaMemcpyHostToDevice) == cudaSuccess;
         ok = ok && cudaMemcpy(s->dpoly, s->poly, sizeof(double) * kPolyTerms, cudaMemcpyHostToDevice) == cudaSuccess;
     }
     std::vector<float> h(kParams);
@@ -1271,9 +1311,8 @@ int amfrw_surrogate_grad(amfrw_surrogate* s, int32_t member, const float* x_norm
         return sg_fail(AMFRW_EINVAL, "bad argument");
     if (rows < 16 || rows > kTrainRows || rows % 16) return sg_fail(AMFRW_EINVAL, "rows must be a multiple of 16 in [16, 1024]");
     cudaStream_t st = s->stream;
-    float *d_x = nullptr, *d_t = nullptr;
-    SG_CUDA(cudaMalloc(&d_x, sizeof(float) * rows * kIn));
-    SG_CUDA(cudaMalloc(&d_t, sizeof(float) * rows));
+    // (the prediction chunk's buffers hold the batch: one pass at a time uses them)
+    float *d_x = s->pz, *d_t = s->ys;
     cudaMemcpyAsync(d_x, x_norm, sizeof(float) * rows * kIn, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_t, targets, sizeof(float) * rows, cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(s->w.loss, 0, sizeof(float), st);
@@ -1286,8 +1325,6 @@ int amfrw_surrogate_grad(amfrw_surrogate* s, int32_t member, const float* x_norm
         if (loss_out) cudaMemcpyAsync(loss_out, s->w.loss, sizeof(float), cudaMemcpyDeviceToHost, st);
         cudaStreamSynchronize(st);
     }
-    cudaFree(d_x);
-    cudaFree(d_t);
     if (rc != AMFRW_OK) return rc;
     return sg_check_err(s);
 }

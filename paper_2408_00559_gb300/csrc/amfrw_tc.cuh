@@ -4,7 +4,7 @@
 //   C[M x N] = A[M x K] * B[N x K]^T        (both operands K-major, BF16;
 //                                             FP32 accumulation in TMEM)
 //
-// One CTA of 128 threads computes a 128 x BN tile (BN <= 256, a multiple of
+// One CTA of 256 threads computes a 128 x BN tile (BN <= 256, a multiple of
 // 16).  K advances in chunks of 64 through a ring of up to four shared-memory
 // stages filled by TMA: one box of 64 elements of K (128 bytes, the 128-byte
 // swizzle's span) by all rows per operand, in the swizzled K-major layout
@@ -17,8 +17,10 @@
 // them to the stage's "empty" mbarrier; the stage of the previous chunk is
 // refilled with the chunk S ahead as soon as that commit completes, while the
 // current chunk's MMAs run.  A final commit releases the epilogue: every warp
-// reads its 32 TMEM lanes (rows) with tcgen05.ld, applies a fused elementwise
-// operation and passes 32 columns at a time through its part of the stages'
+// reads its 32 TMEM lanes (rows; two warps share a quadrant and take its
+// columns in turn, so that the GELU's arithmetic, which bounds the layers, has
+// 16 warps per SM) with tcgen05.ld, applies a fused elementwise operation and
+// passes 32 columns at a time through its part of the stages'
 // memory, so that global accesses are whole 128-byte lines (64 bytes for the
 // BF16 outputs) instead of a sector per row.  Every mbarrier wait is bounded:
 // on timeout the kernel records an error, waits (bounded) once more for the
@@ -36,7 +38,7 @@ namespace tc {
 
 constexpr int kBM = 128;
 constexpr int kBK = 64;
-constexpr int kThreads = 128;
+constexpr int kThreads = 256;
 constexpr uint32_t kSpinLimit = 1u << 26;  // bounded mbarrier waits
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -160,6 +162,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
 // TMEM address.  A stage's operand is one box of rows x 128 bytes.  (1 KB more
 // than needed, to start on a 1024-byte boundary.)
 constexpr int kMaxStages = 4;
+constexpr int kTurnBytes = 32 * 144;  // a warp's buffer in the epilogue
 constexpr int kTileA = kBM * kBK * 2;
 __host__ __device__ constexpr int stage_bytes(int BN) { return kTileA + BN * kBK * 2; }
 __host__ __device__ constexpr int smem_bytes(int BN, int stages) { return 1024 + stages * stage_bytes(BN) + 8 * (2 * kMaxStages + 1) + 16; }
@@ -182,6 +185,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
 struct Epi {
     int mode;             // 0: C = acc (FP32); 1: Z = acc + bias, H = gelu(Z) (BF16), Ht
                           // 2: D = acc * gelu'(Zprev) -> BF16 D and Dt
+                          // 3: y = sum over the 256 columns of w4 * bf16(gelu(acc + bias)), + b4
     float* C;             // mode 0: [M x N] FP32, row stride ldc
     int ldc;
     const float* bias;    // mode 1: [N]
@@ -190,6 +194,8 @@ struct Epi {
     __nv_bfloat16* Ht;    // mode 1/2: [N x M] BF16 transpose (row stride ldt), may be null
     int ldt;
     const float* Zprev;   // mode 2: [M x N] FP32 pre-activation of this layer
+    const float* w4;      // mode 3: [N] (N = BN = 256), then the output's bias b4
+    float* y;             // mode 3: [M]
     int* error;           // set when a bounded wait gave up
 };
 
@@ -206,7 +212,7 @@ __device__ __forceinline__ float gelu_grad(float z)
 }
 
 // C-tile = A[m0:m0+128, :] * B[n0:n0+BN, :]^T; grid (M/128, N/BN).
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 2)
     gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M,
                      int N, int K, int BN, int S, Epi epi)
 {
@@ -300,8 +306,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // turns its 32 x 32 values there, rows 144 bytes apart (FP32) or 80
         // (BF16), so that both the row-wise and the line-wise 16-byte
         // accesses are free of bank conflicts.
-        const int lane = tid & 31, r0 = m0 + warp * 32, row = r0 + lane;
-        unsigned char* tr = smem + warp * 32 * 144;
+        const int lane = tid & 31, quad = warp & 3, half = warp >> 2, r0 = m0 + quad * 32, row = r0 + lane;
+        unsigned char* tr = smem + warp * kTurnBytes;
+        const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16);
         const bool vec_c = (epi.ldc & 3) == 0 && ((uintptr_t)epi.C & 15) == 0;
         auto put_f32 = [&](const float (&v)[32]) {
 #pragma unroll
@@ -320,10 +327,47 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             __syncwarp();
         };
-        for (int c32 = 0; c32 < BN; c32 += 32) {
+        if (epi.mode == 3) {
+            // The output layer on the spot: partial sum l of a row runs over
+            // the columns l, l + 32, ..., then the 32 partial sums are added
+            // pairwise (l and l + 16, then l + 8, ...).  A warp of the
+            // quadrant's pair holds 16 of them; the second hands its over.
+            float part[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) part[i] = 0.0f;
+            for (int c32 = half * 16; c32 < BN; c32 += 32) {
+                float a8[8];
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    tmem_ld8(tq + (uint32_t)(c32 + 8 * g), a8);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int col = c32 + 8 * g + i;
+                        const float h = __bfloat162float(__float2bfloat16(gelu(a8[i] + epi.bias[col])));
+                        part[8 * g + i] = fmaf(h, epi.w4[col], part[8 * g + i]);
+                    }
+                }
+            }
+            float* ex = reinterpret_cast<float*>(smem) + quad * 32 * 17 + lane * 17;
+            if (half == 1) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) ex[i] = part[i];
+            }
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
+            if (half == 0 && row < M) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) part[i] += ex[i];
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (i < o) part[i] += part[i + o];
+                epi.y[row] = part[0] + epi.w4[BN];
+            }
+        } else for (int c32 = half * 32; c32 < BN; c32 += 64) {
             // (a 16-column tile's last 16 values are not read)
             float w[32];
-            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c32;
+            const uint32_t ta = tq + (uint32_t)c32;
             const int nc = BN - c32 < 32 ? 16 : 32, col0 = n0 + c32;
             if (nc == 32) {
                 tmem_ld32(ta, w);
