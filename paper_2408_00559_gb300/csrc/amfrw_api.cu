@@ -275,6 +275,7 @@ struct LaunchClass {
     int kind;            // kWarpGroup, kCtaGroup or kMemGroup
     int item_begin, item_count;
     int block, grid;
+    int csize;           // FP64 CTA and global-memory groups: blocks per grid (grid: clusters)
     size_t smem;
     int smem_group;
     int glog;            // warp groups: log2 lanes per group
@@ -362,6 +363,7 @@ struct Plan {
     int64_t blu_len = 0, blu_cap = 0;
     bool use_multi = true;  // launch strategy (the autotuner may switch it)
     int glog_delta = 0;     // warp groups: lanes per grid widened by 2^glog_delta (autotuned)
+    bool lean = false;      // no spare global scratch (plan_host)
     bool shared_u = false;  // d_u belongs to another plan (the FP64 re-solve writes there)
     const int32_t* inst_mask = nullptr;  // instances to solve, or null for all
 
@@ -401,9 +403,10 @@ int log2i(int v)
 // Host-side plan: validated instances, grid list grouped into launch classes
 // (largest grids first), launch shapes and the size of the line-solve scratch.
 // No device memory is touched.
-// bundles: whether grids may be solved as bundles; bundle_scratch: whether those
-// may keep line-solve factors in global scratch.
-int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool bundle_scratch, Plan& P)
+// bundles: whether grids may be solved as bundles; spare_scratch: false where
+// global scratch is scarce (amfrw_solve_noalloc): bundles then keep no factors
+// there and FP64 grids on whole blocks the smallest slices.
+int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool spare_scratch, Plan& P)
 {
     if (n < 1) return fail(AMFRW_EINVAL, "need at least one instance");
     if (!ps) return fail(AMFRW_EINVAL, "params is NULL");
@@ -415,6 +418,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
             return st;
         }
     }
+    const bool lean = P.lean = !spare_scratch;
     P.n_inst = n;
     const int smem_cap = max_smem_optin();
     // The grids of one instance shape (N, level, psi, full grid, precision,
@@ -449,11 +453,19 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                                          warp ? warp_group_log(llog, mixed) : 5);
                 // grids beyond shared memory, or with lines longer than the register
                 // sweeps take, keep their state in global memory
-                if (force_mem || lay.total > smem_cap || (!warp && maxlv > 5 + rows_log(kCtaGroup, mixed))) {
+                int bytes = lay.total;
+                if (!warp && !mixed) {  // FP64 on whole blocks: lines of any length
+                    bytes = f64_layout(N, g.lv, kCtaGroup, 1, lean).smem;
+                    if (force_mem || bytes > std::min(smem_cap, kF64SmemMax)) {
+                        kind = kMemGroup;
+                        bytes = 0;
+                    }
+                } else if (force_mem || lay.total > smem_cap || (!warp && maxlv > 5 + rows_log(kCtaGroup, mixed))) {
                     kind = kMemGroup;
                     lay = make_layout(N, g.lv, mixed, kind, log2i(kMemBlock));
+                    bytes = lay.total;
                 }
-                gi.push_back(GridInfo{g, lay.L, kind, warp, lay.total, 0});
+                gi.push_back(GridInfo{g, lay.L, kind, warp, bytes, 0});
             }
             it = shapes.emplace(id, std::move(gi)).first;
         }
@@ -561,6 +573,32 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                 return fail(AMFRW_ETOOBIG, "warp groups of a launch class do not fit in shared memory");
             c.block = 32 * wpb;
             c.smem = (size_t)gmax * gpw * wpb;
+        } else if (!c.mixed) {
+            // FP64 on whole blocks: a thread per node up to 256; where there
+            // are fewer grids than SMs, clusters of up to eight blocks per
+            // grid, as long as a block keeps enough nodes to pay for the
+            // barriers (a 65x65 grid on 1, 2, 4, 8 blocks: 190, 137,
+            // 89, 48 us a step)
+            const bool mem = c.kind == kMemGroup;
+            int b = 64;
+            while (b < kCtaMaxThreads && b < lmax) b *= 2;
+            c.block = b;
+            c.csize = 1;
+            int rows = 1 << 30;  // of the axis a cluster splits, and lines along it: a share for every block
+            for (size_t q = k; q < e; ++q) {
+                const int lx = all[q].it.lv[f64_split(c.N, all[q].it.lv)];
+                rows = std::min(rows, std::min(1 << lx, all[q].L >> lx));
+            }
+            while (c.csize < kMaxCluster && c.item_count * c.csize * 2 <= sms && c.csize * 2 <= rows &&
+                   lmax / (c.csize * 2) >= (mem ? 1024 : 128))
+                c.csize *= 2;
+            int bytes = 0;
+            for (size_t q = k; q < e; ++q) {
+                const F64Layout y = f64_layout(c.N, all[q].it.lv, c.kind, c.csize, lean);
+                bytes = std::max(bytes, y.smem);
+                lumax = std::max(lumax, y.slice);
+            }
+            c.smem = mem ? 0 : (size_t)bytes;
         } else if (c.kind == kCtaGroup) {
             int b = 64;
             while (b < kCtaMaxThreads && b * 8 < lmax) b *= 2;
@@ -581,7 +619,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                                            std::to_string(c.smem) + " bytes)");
         const int groups_per_block = c.warp ? (c.block >> c.glog) : 1;
         const int need = (c.item_count + groups_per_block - 1) / groups_per_block;
-        c.grid = std::max(1, std::min(need, per_sm * sms));
+        c.grid = std::max(1, std::min(need, per_sm * sms / std::max(1, c.csize)));
         c.lu_stride = (lumax + 255) & ~(int64_t)255;
         if (c.kind == kMemGroup && c.lu_stride > 0)
             c.grid = (int)std::max<int64_t>(1, std::min<int64_t>(c.grid, kMemScratchBudget / c.lu_stride));
@@ -610,7 +648,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                         bytes = std::max(bytes, y.total);
                         lu = std::max(lu, y.lu < 0 ? y.nlu : 0);
                     }
-                    if (bytes > bundle_budget(c.mixed, lmax) || (lu > 0 && !bundle_scratch)) {
+                    if (bytes > bundle_budget(c.mixed, lmax) || (lu > 0 && !spare_scratch)) {
                         take = 0;
                     } else {
                         c.bundle_smem = std::max(c.bundle_smem, (bytes / nw + 255) & ~255);
@@ -928,6 +966,8 @@ SolveArgs class_args(const Plan& P, const LaunchClass& L, int c, int steps, int 
     a.lu_scratch = P.d_lu ? P.d_lu + L.lu_offset : nullptr;
     a.lu_stride = L.lu_stride;
     a.inst_mask = P.inst_mask;
+    a.csize = std::max(1, L.csize);
+    if (P.lean) a.flags |= kLeanScratch;
     return a;
 }
 
@@ -1017,12 +1057,14 @@ int class_to_global(Plan& P, int c)
     if (L.kind != kCtaGroup) return AMFRW_OK;
     int64_t lumax = 0;
     for (int q = L.item_begin; q < L.item_begin + L.item_count; ++q) {
-        const Layout lay = make_layout(L.N, P.items[(size_t)q].lv, L.mixed, kMemGroup, log2i(kMemBlock));
-        lumax = std::max<int64_t>(lumax, lay.total);
+        const int8_t* lv = P.items[(size_t)q].lv;
+        lumax = std::max<int64_t>(lumax, L.mixed ? make_layout(L.N, lv, true, kMemGroup, log2i(kMemBlock)).total
+                                                 : f64_layout(L.N, lv, kMemGroup, 1, P.lean).slice);
     }
     const int per_sm = occ_for(L.N)(L.mixed, kMemGroup, kMemBlock, 0);
     if (per_sm < 1) return fail(AMFRW_ETOOBIG, "no resident block possible for a global-memory class");
     L.kind = kMemGroup;
+    L.csize = 1;
     L.block = kMemBlock;
     L.smem = 0;
     L.lu_stride = (lumax + 255) & ~(int64_t)255;

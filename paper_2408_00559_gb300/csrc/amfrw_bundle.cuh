@@ -1127,79 +1127,4 @@ __global__ void __launch_bounds__(kBundleThreads, MIXED ? 2 : 1) bundle_kernel(B
     }
 }
 
-// Host launch / occupancy helpers, instantiated once per N.
-template <int N>
-const void* kernel_for(bool mixed, int kind)
-{
-    if (kind == kBundle) return mixed ? (const void*)bundle_kernel<N, true> : (const void*)bundle_kernel<N, false>;
-    if (kind == kWarpGroup)
-        return mixed ? (const void*)solve_kernel<N, true, kWarpGroup> : (const void*)solve_kernel<N, false, kWarpGroup>;
-    if (kind == kCtaGroup)
-        return mixed ? (const void*)solve_kernel<N, true, kCtaGroup> : (const void*)solve_kernel<N, false, kCtaGroup>;
-    return mixed ? (const void*)solve_kernel<N, true, kMemGroup> : (const void*)solve_kernel<N, false, kMemGroup>;
-}
-
-template <int N>
-int launch_impl(const SolveArgs& a, bool mixed, int kind, int block, int grid, size_t smem, void* stream)
-{
-    cudaStream_t st = (cudaStream_t)stream;
-    if (kind == kWarpGroup) {
-        if (mixed) solve_kernel<N, true, kWarpGroup><<<grid, block, smem, st>>>(a);
-        else solve_kernel<N, false, kWarpGroup><<<grid, block, smem, st>>>(a);
-    } else if (kind == kCtaGroup) {
-        if (mixed) solve_kernel<N, true, kCtaGroup><<<grid, block, smem, st>>>(a);
-        else solve_kernel<N, false, kCtaGroup><<<grid, block, smem, st>>>(a);
-    } else {
-        if (mixed) solve_kernel<N, true, kMemGroup><<<grid, block, smem, st>>>(a);
-        else solve_kernel<N, false, kMemGroup><<<grid, block, smem, st>>>(a);
-    }
-    return (int)cudaGetLastError();
-}
-
-template <int N>
-int launch_bundle_impl(const BundleArgs& a, bool mixed, int grid, size_t smem, void* stream)
-{
-    if (mixed) bundle_kernel<N, true><<<grid, kBundleThreads, smem, (cudaStream_t)stream>>>(a);
-    else bundle_kernel<N, false><<<grid, kBundleThreads, smem, (cudaStream_t)stream>>>(a);
-    return (int)cudaGetLastError();
-}
-
-template <int N>
-int occupancy_impl(bool mixed, int kind, int block, size_t smem)
-{
-    int nb = 0;
-    const void* f = kernel_for<N>(mixed, kind);
-    // The limit is an attribute of the kernel, shared by all its launches, and
-    // launches of one kernel request different amounts: past the default
-    // 48 KB, allow the device's opt-in maximum (less the kernel's static
-    // shared memory), so that no launch depends on which query came last.
-    if (smem > 48 * 1024) {
-        int dev = 0, optin = 0;
-        cudaFuncAttributes fa{};
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-            cudaFuncGetAttributes(&fa, f) != cudaSuccess)
-            return 0;
-        const int lim = optin - (int)fa.sharedSizeBytes;
-        if ((size_t)lim < smem ||
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess)
-            return 0;
-    }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem) != cudaSuccess) return 0;
-    return nb;
-}
-
 }  // namespace amfrw
-
-#define AMFRW_INSTANTIATE(NN)                                                               \
-    namespace amfrw {                                                                       \
-    int launch_n##NN(const SolveArgs& a, bool m, int k, int b, int g, size_t s, void* st)   \
-    {                                                                                       \
-        return launch_impl<NN>(a, m, k, b, g, s, st);                                       \
-    }                                                                                       \
-    int launch_bundle_n##NN(const BundleArgs& a, bool m, int g, size_t s, void* st)         \
-    {                                                                                       \
-        return launch_bundle_impl<NN>(a, m, g, s, st);                                      \
-    }                                                                                       \
-    int occupancy_n##NN(bool m, int k, int b, size_t s) { return occupancy_impl<NN>(m, k, b, s); } \
-    }

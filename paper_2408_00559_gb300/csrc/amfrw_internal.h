@@ -325,10 +325,126 @@ struct SolveArgs {
     // instances to solve (nonzero entries), or null for all: the FP64
     // re-solve of ill-conditioned mixed-precision instances skips the others
     const int32_t* inst_mask;
+    int32_t csize;        // FP64 CTA and global-memory groups: blocks per grid (a cluster)
 };
 
 constexpr int kLoadState = 1;
 constexpr int kStoreState = 2;
+constexpr int kLeanScratch = 4;  // FP64 global-memory groups: the smallest slices
+
+// FP64 grids on whole blocks (amfrw_f64.cuh): offsets of a grid's arrays.  CTA
+// groups keep the vectors the stencil reads (Z, K1, Kw) and the small tables in
+// shared memory, then what fits of the central differences (single blocks),
+// the right-hand sides K0 (clusters: their barriers empty the L1 cache), the
+// line-solve factors and the tables by rate index, the rest in the slice of
+// global scratch; global-memory groups keep everything there.
+constexpr int kF64SmemMax = 224 * 1024;
+constexpr int kMaxCluster = 8;
+
+// log2 of the lanes among which the lines of a solve are spread: all warps of
+// a block; half of a cluster's, whose lines are short enough by then (65x65
+// grid on eight blocks: 1.25 ms with a quarter, 1.04 with half).
+AMFRW_HD int f64_tlog(int csize)
+{
+    int c = 0;
+    while ((2 << c) <= csize) ++c;
+    return 8 + (c > 0 ? c - 1 : 0);
+}
+
+struct F64Layout {
+    int32_t Lp, diff;
+    int32_t cst, tabd, pay, cxt, Z, K1, Kw, D, scr;  // in shared memory (global-memory groups: in the slice)
+    int32_t lu, H, dr, K0;                           // in the slice, or (bits of `fast`) in shared memory
+    int32_t fast;                                    // 1 lu, 2 H, 4 dr, 8 K0
+    int32_t smem;
+    int64_t slice;
+};
+
+// A cluster splits a grid along its longest axis (the last of equal ones):
+// each block owns a slab of its rows.
+AMFRW_HD int f64_split(int N, const int8_t* lv)
+{
+    int x = 0;
+    for (int i = 1; i < N; ++i)
+        if (lv[i] >= lv[x]) x = i;
+    return x;
+}
+// Whether a block meets only its slab's line classes of an axis: two axes split
+// along V, where a line of the rate axis is a class.
+AMFRW_HD bool f64_own_classes(int N, const int8_t* lv, int axis, int csize)
+{
+    return N == 2 && axis == 0 && csize > 1 && f64_split(N, lv) == 1;
+}
+
+AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, bool lean)
+{
+    F64Layout y{};
+    int llog = 0, sumM = 0, npay = 0, ncx = 0;
+    for (int i = 0; i < N; ++i) llog += lv[i];
+    bool rate_rows = false;
+    for (int i = 0; i < N - 1; ++i) {
+        sumM += 1 << lv[i];
+        npay += (1 << lv[i]) + 1;
+        rate_rows |= lv[i] > 0;
+        for (int k = i + 1; k < N; ++k) ncx += k < N - 1 ? 1 << lv[k] : 1;
+    }
+    const int MV = 1 << lv[N - 1], L = 1 << llog, Lr = L >> lv[N - 1];
+    y.Lp = L + ((1 << lv[0]) >= pad_rows_min(false) ? L >> lv[0] : 0);
+    int ndr = 0, sh = 0, rmax = 0;
+    int64_t nlu = 0, nlu_own = 0;  // factor values; those one block of a cluster uses
+    for (int i = 0; i < N; ++i) {
+        const int rows = (i < N - 1 ? MV : 1) << lv[i];
+        rmax = rows > rmax ? rows : rmax;
+        // (make_shape's line-solve region: folded axes keep their place)
+        const int64_t n = (int64_t)rows * lu_row_values(lanes_log(lv[i], llog, f64_tlog(csize), kRowsLogMem));
+        nlu += n;
+        nlu_own += f64_own_classes(N, lv, i, csize) ? n / csize : n;
+        if (i >= 1 && i < N - 1 && lv[i] > 0) ndr += 1 << (sh + lv[i] - lv[0]);
+        sh += lv[i];
+    }
+    const bool mem = kind == kMemGroup;
+    int64_t g = 0;  // the slice
+    int o = 0;      // shared memory
+    auto small = [&](int bytes) {
+        if (mem) {
+            const int64_t at = g;
+            g += (bytes + 15) & ~15;
+            return (int32_t)at;
+        }
+        const int at = o;
+        o = align16(o + bytes);
+        return (int32_t)at;
+    };
+    y.cst = small(8 * (int)(sizeof(Consts<double>) / sizeof(double)));
+    y.tabd = small(8 * (3 * sumM + MV));
+    y.pay = small(8 * 2 * npay);
+    y.cxt = small(8 * ncx);
+    y.Z = small(8 * y.Lp);
+    y.scr = y.Z;  // (at most three vectors: rmax <= L)
+    y.K1 = small(8 * y.Lp);
+    y.Kw = small(8 * y.Lp);
+    const int64_t dbytes = (int64_t)8 * (N - 1) * y.Lp;
+    y.diff = mem ? (lean ? 0 : 1) : (csize == 1 && o + dbytes <= kF64SmemMax ? 1 : 0);
+    y.D = y.diff ? small((int)dbytes) : 0;
+    // in shared memory while it lasts, else in the slice
+    auto rest = [&](int64_t fast_bytes, int64_t bytes, int bit) {
+        if (!mem && o + fast_bytes + 16 <= kF64SmemMax) {
+            y.fast |= bit;
+            return small((int)fast_bytes);
+        }
+        const int64_t at = g;
+        g += (bytes + 15) & ~(int64_t)15;
+        return (int32_t)at;
+    };
+    if (csize > 1) y.K0 = rest((int64_t)8 * y.Lp, (int64_t)8 * y.Lp, 8);
+    y.lu = rest(8 * nlu_own, 8 * nlu, 1);
+    y.H = rest((int64_t)8 * Lr, (int64_t)8 * Lr, 2);
+    y.dr = lean ? 0 : rest((int64_t)8 * ndr, (int64_t)8 * ndr, 4);
+    if (csize == 1) y.K0 = rest((int64_t)8 * y.Lp, (int64_t)8 * y.Lp, 8);
+    y.smem = o;
+    y.slice = (g + 255) & ~(int64_t)255;
+    return y;
+}
 
 // Bundles (amfrw_bundle.cuh): up to 32 grids of one shape, one instance per
 // lane, on a group of warps that share the nodes.

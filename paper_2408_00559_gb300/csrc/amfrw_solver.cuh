@@ -2111,67 +2111,4 @@ __device__ void solve_item_mixed(const SolveArgs& a, const Item& it, unsigned ch
     gsync<WARP>(gm);  // the group's shared memory is reused by its next grid
 }
 
-// The solver kernel.  CTA groups: one grid per block at a time from the
-// launch's work counter.  Warp groups: a persistent multi-class launch -- every
-// warp walks the launch's class list (ordered largest grids first) and takes
-// chunks of 32 >> glog grids from each class's counter until it is exhausted,
-// then moves on, so classes of uneven instances share one launch and no warp
-// waits for another.
-template <int N, bool MIXED, int KIND>
-__global__ void __launch_bounds__(KIND == kWarpGroup ? 128 : kCtaMaxThreads, KIND == kWarpGroup ? (MIXED ? kWarpBlocksMixed : 3) : ((KIND == kMemGroup || MIXED) ? 2 : 1)) solve_kernel(SolveArgs a)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    if constexpr (KIND == kWarpGroup) {
-        const int warp = threadIdx.x >> 5;
-        const int lane = threadIdx.x & 31;
-        unsigned char* wbase = smem + (size_t)warp * (size_t)a.smem_warp;
-        int c = 0;
-        while (c < a.n_classes) {
-            const ClassDesc cd = a.classes[c];
-            int chunk = 0;
-            if (lane == 0) chunk = atomicAdd(a.queue + cd.qidx, 32 >> cd.glog);
-            chunk = __shfl_sync(0xffffffffu, chunk, 0);
-            if (chunk >= cd.item_count) {
-                ++c;
-                continue;
-            }
-            const int item = chunk + (lane >> cd.glog);
-            bool take = item < cd.item_count;
-            Item it{};
-            if (take) {
-                it = a.items[cd.item_begin + item];
-                take = !a.inst_mask || a.inst_mask[it.inst] != 0;
-            }
-            if (take) {
-                const int gsize = 1 << cd.glog;
-                unsigned char* base = wbase + (size_t)(lane >> cd.glog) * (size_t)cd.smem_group;
-                if constexpr (MIXED)
-                    solve_item_mixed<N, kWarpGroup>(a, it, base, base, lane & (gsize - 1), gsize);
-                else
-                    solve_item<N, false, kWarpGroup>(a, it, base, lane & (gsize - 1), gsize);
-            }
-        }
-    } else {
-        // CTA groups: the grid in shared memory; global-memory groups: in the
-        // block's slice of the scratch array
-        unsigned char* base = KIND == kMemGroup ? a.lu_scratch + (size_t)blockIdx.x * (size_t)a.lu_stride : smem;
-        __shared__ int s_item;
-        for (;;) {
-            if (threadIdx.x == 0) s_item = atomicAdd(a.queue, 1);
-            __syncthreads();
-            const int item = s_item;
-            __syncthreads();
-            if (item >= a.n_items) break;
-            const Item it = a.items[item];
-            if (a.inst_mask && a.inst_mask[it.inst] == 0) continue;  // uniform across the block
-            // whole-block groups keep the unrolled stencil of solve_item in both
-            // precisions: with up to 256 threads on one grid the per-node work
-            // dominates, and the unrolled form, each axis's offsets in
-            // registers, measured 30 % faster on the d=6 modified level-6
-            // workload than the table-driven form of the warp groups
-            solve_item<N, MIXED, KIND>(a, it, base, (int)threadIdx.x, (int)blockDim.x);
-        }
-    }
-}
-
 }  // namespace amfrw
