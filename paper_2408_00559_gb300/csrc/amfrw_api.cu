@@ -792,9 +792,37 @@ int build_warp_launches(Plan& P)
             items += d.item_count << d.glog;  // lanes of work
         }
         if (w.cls.empty()) continue;
+        // A launch that leaves most of the chip idle (one instance) is as slow
+        // as its longest grid: FP64 grids then get up to all 32 lanes each (a
+        // node per lane instead of two, so half the instructions per lane; a d=4
+        // level-5 instance of 121 grids, 40 steps: 1.00 -> 0.73 ms).  The line
+        // is a warp per scheduler, where more lanes no longer come for free.
+        // Mixed precision keeps its widths, which fix the roundings of long
+        // lines.
+        if (!w.mixed) {
+            auto lanes = [&](int wider) {
+                int64_t v = 0;
+                for (const ClassDesc& d : w.cls) v += (int64_t)d.item_count << std::min(5, d.glog + wider);
+                return v;
+            };
+            int wider = 0;
+            while (wider < 2 && lanes(wider + 1) <= (int64_t)sms * 128) ++wider;
+            if (wider > 0) {
+                items = (int)lanes(wider);
+                w.smem_warp = 0;
+                for (ClassDesc& d : w.cls) {
+                    const LaunchClass& L = P.classes[(size_t)(d.qidx)];
+                    d.glog = std::min(5, d.glog + wider);
+                    d.smem_group = group_smem_of(P, L, d.glog);
+                    w.smem_warp = std::max(w.smem_warp, d.smem_group << (5 - d.glog));
+                }
+            }
+        }
         if (w.smem_warp > smem_cap)
             return fail(AMFRW_ETOOBIG, "the work groups of one warp do not fit in shared memory");
-        const int wpb = std::min(kWarpsPerBlock, std::max(1, smem_cap / w.smem_warp));
+        // (few warps: a block each, so that they spread over the SMs)
+        int wpb = std::min(kWarpsPerBlock, std::max(1, smem_cap / w.smem_warp));
+        while (wpb > 1 && (items + 31) / 32 <= sms * (wpb / 2)) wpb /= 2;
         w.block = 32 * wpb;
         w.smem = (size_t)w.smem_warp * wpb;
         const int per_sm = occ_for(w.N)(w.mixed, kWarpGroup, w.block, w.smem);
