@@ -159,6 +159,11 @@ __device__ __forceinline__ void block_F(const unsigned char* sm, int pc, int n, 
     };
     auto top = [&](int a, int k) -> bool { return SEG ? (k == NB - 1 && seg_last) : row(a, k) == P_::M(a) - 1; };
 
+    // p - 2 x + m from g = p - m; without a row below (m = 0), g is not used.
+    // (Neighbour sums with a centre coefficient take an operation less, but
+    // cancel: they serve the axes of one and two rows.)
+    auto second = [](T p, T xv, T g, bool lo) -> T { return lo ? fma(T(2), p - xv, -g) : fma(T(-2), xv, p); };
+
     // axis q, the inner axis A
     auto inner_axis = [&](auto Ac, int4 h) {
         constexpr int a = decltype(Ac)::value;
@@ -173,12 +178,13 @@ __device__ __forceinline__ void block_F(const unsigned char* sm, int pc, int n, 
             if constexpr (SUM) {
                 const bool lo = SEG ? (k > 0 || seg_lo) : row(a, k) > 0;
                 if (top(a, k)) {
-                    acc[k] = fma(T(2) * d, Src::val(m), acc[k]);
+                    acc[k] = fma(T(2) * d, SEG ? Src::val(m) - Src::val(x[k]) : Src::val(m), acc[k]);
                     grad[k] = T(0);
                 } else {
                     const T p = Src::val(up(a, k, x, xp));
-                    acc[k] = fma(d, lo ? p + Src::val(m) : p, acc[k]);
                     grad[k] = lo ? p - Src::val(m) : p;
+                    if (SEG) acc[k] = fma(d, second(p, Src::val(x[k]), grad[k], lo), acc[k]);
+                    else acc[k] = fma(d, lo ? p + Src::val(m) : p, acc[k]);
                 }
             } else {
                 const V p = top(a, k) ? m : up(a, k, x, xp);
@@ -262,21 +268,21 @@ __device__ __forceinline__ void block_F(const unsigned char* sm, int pc, int n, 
             if (lo) load(h.w, Q);
             if (h.x & (kBlkTop << 8)) {
 #pragma unroll
-                for (int k = 0; k < NB; ++k) acc[k] = fma(T(2) * d, Src::val(Q[k]), acc[k]);
+                for (int k = 0; k < NB; ++k) acc[k] = fma(T(2) * d, Src::val(Q[k]) - Src::val(x[k]), acc[k]);
                 return;
             }
             load(h.z, P);
             if (lo) {
 #pragma unroll
                 for (int k = 0; k < NB; ++k) {
-                    acc[k] = fma(d, Src::val(P[k]) + Src::val(Q[k]), acc[k]);
                     grad[k] = Src::val(P[k]) - Src::val(Q[k]);
+                    acc[k] = fma(d, second(Src::val(P[k]), Src::val(x[k]), grad[k], true), acc[k]);
                 }
             } else {
 #pragma unroll
                 for (int k = 0; k < NB; ++k) {
                     grad[k] = Src::val(P[k]);
-                    acc[k] = fma(d, grad[k], acc[k]);
+                    acc[k] = fma(d, second(grad[k], Src::val(x[k]), T(0), false), acc[k]);
                 }
             }
         } else {
@@ -729,10 +735,18 @@ __device__ void bundle_build(unsigned char* sm, unsigned char* lub, const Bundle
     }
     if (w == 0) tab[y.cv * 32] = (T)cV;
     if constexpr (!MIXED) {
-        // centre coefficients by rate index
+        // centre coefficients by rate index, of the axes of one row and the
+        // block's axes of two
+        auto centred = [&](int i) {
+            bool c = s.M[i] == 1;
+            if (y.pat != kPatSeg)
+                for (int b = 0; b < (y.pat == kPat22 ? 2 : (y.pat == kPat2 ? 1 : 0)); ++b) c |= y.ax[y.in[b]] == i;
+            return c;
+        };
         for (int t = w; t < y.Lr; t += W) {
-            double sum = cV;
-            for (int i = 0; i < N - 1; ++i) sum += tab[(s.toff[i] + ((t >> s.sh[i]) & (s.M[i] - 1))) * 32];
+            double sum = centred(N - 1) ? cV : 0.0;
+            for (int i = 0; i < N - 1; ++i)
+                if (centred(i)) sum += tab[(s.toff[i] + ((t >> s.sh[i]) & (s.M[i] - 1))) * 32];
             tab[(y.c0 + t) * 32] = -2.0 * sum;
         }
     }
