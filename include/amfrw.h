@@ -93,7 +93,7 @@ enum amfrw_precision {
  *   flags     bitwise or of
  *             AMFRW_FLAG_GLOBAL_GRIDS: solve every component grid with its
  *               state in global memory, the path that grids too large for
- *               shared memory (or with lines of more than 256 rows) always
+ *               shared memory (or, mixed, with lines of more than 128 rows) always
  *               take; the result is the same to rounding;
  *             AMFRW_FLAG_DIRICHLET: the earlier boundary conditions of eq.
  *               bound1_0 instead of the Neumann faces of eq. bound1 on the

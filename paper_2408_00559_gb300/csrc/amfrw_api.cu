@@ -465,8 +465,8 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                 int kind = warp ? kWarpGroup : kCtaGroup;
                 Layout lay = make_layout(N, g.lv, mixed, kind,
                                          warp ? warp_group_log(llog, mixed) : 5);
-                // grids beyond shared memory, or with lines longer than the register
-                // sweeps take, keep their state in global memory
+                // grids beyond shared memory, or (mixed) with lines longer than
+                // the register sweeps take, keep their state in global memory
                 int bytes = lay.total;
                 if (!warp && !mixed) {  // FP64 on whole blocks: lines of any length
                     bytes = f64_layout(N, g.lv, kCtaGroup, 1, lean).smem;
@@ -474,7 +474,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                         kind = kMemGroup;
                         bytes = 0;
                     }
-                } else if (force_mem || lay.total > smem_cap || (!warp && maxlv > 5 + rows_log(kCtaGroup, mixed))) {
+                } else if (force_mem || lay.total > smem_cap || (!warp && maxlv > 5 + rows_log(kCtaGroup))) {
                     kind = kMemGroup;
                     lay = make_layout(N, g.lv, mixed, kind, log2i(kMemBlock));
                     bytes = lay.total;

@@ -117,33 +117,27 @@ AMFRW_HD constexpr int shape_bytes(int N) { return align16(4 * (10 * N + 8)); }
 AMFRW_HD constexpr int meta_bytes(int N) { return shape_bytes(N) + align16((int)sizeof(ActAxes)); }
 constexpr int kMetaBytesMax = meta_bytes(kMaxDim);
 
-// Work-group kinds.  kBundle: grids of at most 64 Inner nodes of many
-// instances, one instance per lane.  kWarpGroup: a grid of at most 64 Inner nodes on (part
-// of) one warp, everything in shared memory.  kCtaGroup: one CTA per grid,
-// the grid in shared memory, line-solve factors in a global scratch slice.
-// kMemGroup: one CTA per grid with the whole grid state in its block's slice
-// of global scratch (L2/HBM resident): grids too large for shared memory or
-// with lines of more than 256 rows.
+// Work-group kinds.  kBundle: grids of one shape of many instances, one instance
+// per lane.  kWarpGroup: a grid of at most 64 Inner nodes on (part of) one warp,
+// everything in shared memory.  kCtaGroup: one CTA per grid (FP64: or a cluster
+// of them), the grid in shared memory, line-solve factors there or in a global
+// scratch slice.  kMemGroup: the same with the whole grid state in a slice of
+// global scratch (L2/HBM resident): grids too large for shared memory or, in
+// mixed precision, with lines of more than 128 rows.
 constexpr int kWarpGroup = 0;
 constexpr int kCtaGroup = 1;
 constexpr int kMemGroup = 2;
 constexpr int kBundle = 3;
 
 // Rows of a line per lane in a line solve: at most 2 for warp groups (grids of
-// at most 64 Inner nodes), at most 8 for FP64 CTA groups and 4 for
-// mixed-precision ones (rows held in registers; mixed-precision CTA groups
-// run two blocks per SM, so 128 registers a thread), hence lines of at most
-// 256 / 128 rows there; unbounded for global-memory groups (rows streamed
-// from memory).
+// at most 64 Inner nodes) and 4 for mixed-precision CTA groups (rows held in
+// registers; they run two blocks per SM, so 128 registers a thread), hence
+// lines of at most 128 rows there; unbounded for global-memory groups and FP64
+// CTA groups (rows streamed from memory).
 constexpr int kRowsLogWarp = 1;
-constexpr int kRowsLogCta = 3;
-constexpr int kRowsLogCtaMixed = 2;
+constexpr int kRowsLogCta = 2;
 constexpr int kRowsLogMem = 24;
-AMFRW_HD int rows_log(int kind, bool mixed = false)
-{
-    return kind == kWarpGroup ? kRowsLogWarp
-                              : (kind == kCtaGroup ? (mixed ? kRowsLogCtaMixed : kRowsLogCta) : kRowsLogMem);
-}
+AMFRW_HD int rows_log(int kind) { return kind == kWarpGroup ? kRowsLogWarp : (kind == kCtaGroup ? kRowsLogCta : kRowsLogMem); }
 
 // Lanes per line (as log2) for the directional solves along an axis with
 // 2^mlog rows, on a grid of 2^llog Inner nodes solved by a group of 2^tlog
@@ -221,7 +215,7 @@ AMFRW_HD Layout make_layout(int N, const int8_t* lv, bool mixed, int kind, int t
             nlu = (nlu + 3) & ~3;
             nlu += rows << lv[i];
         } else {
-            nlu += rows * lu_row_values(lanes_log(lv[i], llog, tlog, rows_log(kind, mixed)));
+            nlu += rows * lu_row_values(lanes_log(lv[i], llog, tlog, rows_log(kind)));
         }
     }
     const bool lu_in = kind != kCtaGroup;

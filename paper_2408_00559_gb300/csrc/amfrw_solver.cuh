@@ -1207,8 +1207,7 @@ __device__ __forceinline__ void lsweep(const Shape<N>& s, int axis, const T* __r
                                        const T* src, T* dst, int rank, int gsize, unsigned gm,
                                        Epi epi)
 {
-    constexpr int RM = 1 << (KIND == kWarpGroup ? kRowsLogWarp
-                                                : (std::is_same<T, float>::value ? kRowsLogCtaMixed : kRowsLogCta));
+    constexpr int RM = 1 << (KIND == kWarpGroup ? kRowsLogWarp : kRowsLogCta);
     if constexpr (KIND == kMemGroup)
         sweep_mem<N, T>(s, axis, lu, src, dst, rank, gsize, gm, epi);
     else if constexpr (N <= 4)
@@ -1472,14 +1471,16 @@ __device__ __forceinline__ void interp_spot(const Shape<N>& s, const InstDev& P,
 }
 
 // ------------------------------------------------------------- one grid
+// FP64 on warp groups, mixed precision on CTA and global-memory groups.
 template <int N, bool MIXED, int KIND>
 __device__ void solve_item(const SolveArgs& a, const Item& it, unsigned char* base, int rank,
                            int gsize)
 {
     using TK = typename std::conditional<MIXED, float, double>::type;
     constexpr bool WARP = KIND == kWarpGroup;
+    static_assert(MIXED != WARP);
     const InstDev& P = a.insts[it.inst];
-    constexpr int RMAX = 1 << (WARP ? kRowsLogWarp : (MIXED ? kRowsLogCtaMixed : kRowsLogCta));
+    constexpr int RMAX = 1 << (WARP ? kRowsLogWarp : kRowsLogCta);
     const int tlog = 31 - __clz(gsize);
     const unsigned gm = WARP ? group_mask(tlog) : 0xffffffffu;
     Shape<N> s;
@@ -1490,7 +1491,7 @@ __device__ void solve_item(const SolveArgs& a, const Item& it, unsigned char* ba
     // mixed-precision CTA groups keep Z and dt F(Y_n) in their block's global
     // slice and pad fewer rows, so that two CTAs fit an SM's shared memory
     constexpr bool LEAN = MIXED && KIND == kCtaGroup;
-    make_shape<N>(s, it.lv, tlog, rows_log(KIND, MIXED), KIND != kMemGroup, kFoldV, P.bc != 0, false,
+    make_shape<N>(s, it.lv, tlog, rows_log(KIND), KIND != kMemGroup, kFoldV, P.bc != 0, false,
                   pad_rows_min(LEAN));
     const int last = kFoldV ? s.last : N - 1;  // the axis whose solve carries the epilogues
     const Layout lay = make_layout(N, it.lv, MIXED, KIND, tlog);
@@ -1583,21 +1584,13 @@ __device__ void solve_item(const SolveArgs& a, const Item& it, unsigned char* ba
             const int J = s.padded(t);
             if (dirichlet_node(s, t)) {  // no stencil on a Dirichlet face (its far neighbour is not stored)
                 K0[J] = TK(0);
-                if constexpr (MIXED) FY[J] = 0.f;
+                FY[J] = 0.f;
                 continue;
             }
-            TK k0;
-            if constexpr (MIXED) {
-                const float acc = stencil_acc<N, float>(s, j, J, DFSrc{ZZ}, (const float*)tabk,
-                                                        *(const Consts<float>*)ck);
-                k0 = (TK)(ck->dt * v2[j[N - 1]] * ((float)H[t & Lr1] + acc));
-                FY[J] = (float)k0;
-            } else {
-                const double acc = stencil_acc<N, double>(s, j, J, ArrSrc<double>{Z},
-                                                          (const double*)tabk,
-                                                          *(const Consts<double>*)ck);
-                k0 = (TK)(cd->dt * (double)v2[j[N - 1]] * ((double)H[t & Lr1] + acc));
-            }
+            const float acc = stencil_acc<N, float>(s, j, J, DFSrc{ZZ}, (const float*)tabk,
+                                                    *(const Consts<float>*)ck);
+            const TK k0 = (TK)(ck->dt * v2[j[N - 1]] * ((float)H[t & Lr1] + acc));
+            FY[J] = (float)k0;
             K0[J] = k0;
         }
         gsync<WARP>(gm);
@@ -1666,19 +1659,11 @@ __device__ void solve_item(const SolveArgs& a, const Item& it, unsigned char* ba
                 K0[J] = TK(0);
                 continue;
             }
-            if constexpr (MIXED) {
-                const float acc = stencil_acc<N, float>(s, j, J, ArrSrc<float>{(const float*)K1},
-                                                        (const float*)tabk,
-                                                        *(const Consts<float>*)ck);
-                const float a21dt = (float)kA21 * (float)ck->dt;
-                K0[J] = (TK)(FY[J] + a21dt * (float)v2[j[N - 1]] * acc + (float)kQ21 * (float)K1[J]);
-            } else {
-                const double acc = stencil_acc<N, double>(s, j, J, ArrSrc<double>{(const double*)Kw},
-                                                          (const double*)tabk,
-                                                          *(const Consts<double>*)ck);
-                K0[J] = (TK)(cd->dt * (double)v2[j[N - 1]] * ((double)H[t & Lr1] + acc) +
-                             kQ21 * (double)K1[J]);
-            }
+            const float acc = stencil_acc<N, float>(s, j, J, ArrSrc<float>{(const float*)K1},
+                                                    (const float*)tabk,
+                                                    *(const Consts<float>*)ck);
+            const float a21dt = (float)kA21 * (float)ck->dt;
+            K0[J] = (TK)(FY[J] + a21dt * (float)v2[j[N - 1]] * acc + (float)kQ21 * (float)K1[J]);
         }
         gsync<WARP>(gm);
         sweeps_into<N, TK, KIND>(s, luc, K0, Kw, rank, gsize, gm);
@@ -1911,13 +1896,13 @@ __device__ void solve_item_mixed(const SolveArgs& a, const Item& it, unsigned ch
     static_assert(KIND == kWarpGroup, "the register-resident phases need at most two nodes per lane");
     constexpr bool WARP = true;
     const InstDev& P = a.insts[it.inst];
-    constexpr int RMAX = 1 << (WARP ? kRowsLogWarp : kRowsLogCtaMixed);
+    constexpr int RMAX = 1 << (WARP ? kRowsLogWarp : kRowsLogCta);
     const int tlog = 31 - __clz(gsize);
     const unsigned gm = WARP ? group_mask(tlog) : 0xffffffffu;
     Shape<N>& s = *reinterpret_cast<Shape<N>*>(meta);
     ActAxes& A = *reinterpret_cast<ActAxes*>(meta + shape_bytes(N));
     // single-row solves are folded into another solve
-    if (rank == 0) make_shape<N>(s, it.lv, tlog, rows_log(KIND, true), true, true, P.bc != 0, true);
+    if (rank == 0) make_shape<N>(s, it.lv, tlog, rows_log(KIND), true, true, P.bc != 0, true);
     gsync<WARP>(gm);
     const Layout lay = make_layout(N, it.lv, true, KIND, tlog);
     Consts<double>* cd = reinterpret_cast<Consts<double>*>(base + lay.cd);
