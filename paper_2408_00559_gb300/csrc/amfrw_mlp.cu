@@ -62,6 +62,51 @@ int device_sms(int dev)
     return v;
 }
 
+// Columns of a tile.  The widest tile reads A once; where that leaves SMs idle
+// (a training batch has 8 row tiles) narrower ones, down to 32 columns, share
+// the work (A's tiles come from L2).
+int tile_columns(int M, int N, int sms)
+{
+    int BN = N <= 256 ? N : 256;
+    const int rt = (M + kBM - 1) / kBM;
+    while (BN % 32 == 0 && BN > 32 && rt * ((N + BN - 1) / BN) * 2 <= sms) BN /= 2;
+    return BN;
+}
+
+// Stages of a launch of `tiles` blocks.  Two CTAs share an SM when there are
+// more tiles than SMs (at most two stages of the widest tile, 96 KB: one's
+// epilogue overlaps the other's loads and MMAs); else a block may have the SM's
+// shared memory, since a chunk's loads take longer than its MMAs and only loads
+// in flight hide that (one 256 x 256 x 1024 product on 16 blocks took 14.5 us
+// with four stages; the three of a training batch, in one launch with eight,
+// take 12.6).
+int tile_stages(int BN, int nk, int tiles, int sms)
+{
+    int S = kMaxStages;
+    while (S > 1 && (S > nk || smem_bytes(BN, S) > (tiles <= sms ? 200 : 112) * 1024)) --S;
+    return S;
+}
+
+// (the epilogue turns its values through the stages' memory)
+int tile_smem(int BN, int S) { return std::max(smem_bytes(BN, S), 1024 + kThreads / 32 * kTurnBytes); }
+
+// Raises the kernels' dynamic shared-memory limit, an attribute per device,
+// once on every device that launches them (to the most any launch asks for).
+int raise_limits(int dev)
+{
+    static std::mutex mu;
+    static bool attr[64] = {};
+    std::lock_guard<std::mutex> lock(mu);
+    if (!attr[dev]) {
+        const int most = 200 * 1024 + 1024;
+        cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return (int)e;
+        attr[dev] = true;
+    }
+    return 0;
+}
+
 // C[M x N] = A[M x K] * B[N x K]^T with the fused epilogue `epi`; N split in
 // column tiles of at most 256.  A, B: 16-byte aligned, lda and ldb multiples
 // of 8 (the tensor maps' row strides are multiples of 16 bytes).
@@ -72,36 +117,49 @@ int gemm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return (int)e;
     if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
-    // The widest tile reads A once; where that leaves SMs idle (a training
-    // batch has 8 row tiles) narrower ones, down to 32 columns, share the work
-    // (A's tiles come from L2).
-    int BN = N <= 256 ? N : 256;
-    const int rt = (M + kBM - 1) / kBM, sms = device_sms(dev);
-    while (epi.mode != 3 && BN % 32 == 0 && BN > 32 && rt * ((N + BN - 1) / BN) * 2 <= sms) BN /= 2;
-    const int nk = (K + kBK - 1) / kBK;
-    // at most two stages of the widest tile (96 KB), so that two CTAs share an
-    // SM and one's epilogue overlaps the other's loads and MMAs
-    int S = kMaxStages;
-    while (S > 1 && (S > nk || smem_bytes(BN, S) > 112 * 1024)) --S;
-    // (the epilogue turns its values through the stages' memory)
-    const int smem = std::max(smem_bytes(BN, S), 1024 + kThreads / 32 * kTurnBytes);
-    // The dynamic shared-memory limit is a per-device attribute of the
-    // kernel: raise it once on every device that launches it (to the most any
-    // launch asks for).
-    static std::mutex mu;
-    static bool attr[64] = {};
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!attr[dev]) {
-            e = cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024 + 1024);
-            if (e != cudaSuccess) return (int)e;
-            attr[dev] = true;
-        }
-    }
+    const int sms = device_sms(dev);
+    const int BN = epi.mode == 3 ? (N <= 256 ? N : 256) : tile_columns(M, N, sms);
+    const dim3 grid((M + kBM - 1) / kBM, (N + BN - 1) / BN);
+    const int S = tile_stages(BN, (K + kBK - 1) / kBK, grid.x * grid.y, sms);
+    if (const int rc = raise_limits(dev)) return rc;
     CUtensorMap tA, tB;
     if (!make_map(&tA, A, M, K, lda, kBM) || !make_map(&tB, B, N, K, ldb, BN)) return (int)cudaErrorInvalidValue;
-    dim3 grid((M + kBM - 1) / kBM, (N + BN - 1) / BN);
-    gemm_bf16_kernel<<<grid, kThreads, smem, st>>>(tA, tB, M, N, K, BN, S, epi);
+    gemm_bf16_kernel<<<grid, kThreads, tile_smem(BN, S), st>>>(tA, tB, M, N, K, BN, S, epi);
+    return (int)cudaGetLastError();
+}
+
+// Three products C = A B^T of one K (FP32 results), as gemm's, in one launch.
+struct Product {
+    const __nv_bfloat16 *A, *B;
+    float* C;
+    int ldc, M, N;
+};
+int gemm3(const Product (&p)[3], int lda, int ldb, int K, int* error, cudaStream_t st)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return (int)e;
+    if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
+    const int sms = device_sms(dev);
+    Jobs j{};
+    j.K = K;
+    j.error = error;
+    int wide = 0;
+    for (int q = 0; q < 3; ++q) {
+        const int BN = tile_columns(p[q].M, p[q].N, sms);
+        j.C[q] = p[q].C;
+        j.ldc[q] = p[q].ldc;
+        j.M[q] = p[q].M;
+        j.N[q] = p[q].N;
+        j.BN[q] = BN;
+        j.first[q + 1] = j.first[q] + (p[q].M + kBM - 1) / kBM * ((p[q].N + BN - 1) / BN);
+        wide = std::max(wide, BN);
+        if (!make_map(&j.a[q], p[q].A, p[q].M, K, lda, kBM) || !make_map(&j.b[q], p[q].B, p[q].N, K, ldb, BN))
+            return (int)cudaErrorInvalidValue;
+    }
+    j.S = tile_stages(wide, (K + kBK - 1) / kBK, j.first[3], sms);
+    if (const int rc = raise_limits(dev)) return rc;
+    gemm_bf16_batch_kernel<<<j.first[3], kThreads, tile_smem(wide, j.S), st>>>(j);
     return (int)cudaGetLastError();
 }
 
@@ -330,36 +388,45 @@ __global__ void pack_kernel(const float* __restrict__ feats, const float* __rest
     if (c == 0 && t) t[b] = targets[row];
 }
 
-// y_b = H3_b . w4 + b4 (one warp per row).
-__global__ void out_fwd_kernel(const bf16* __restrict__ H3, const float* __restrict__ P, float* y, int B)
+// The output layer and its backward pass: y = H3 . w4 + b4, L = 1/2 mean
+// (y - t)^2 (accumulated into *loss), dy = (y - t)/B, dZ3 = dy w4 gelu'(Z3)
+// (BF16 and its transpose).  A block takes kOutRows rows, a warp one at a time;
+// the transpose goes through shared memory, so that its 16-byte stores fill
+// sectors (a warp per row with two-byte stores B apart: 12.5 us for 1024 rows,
+// this 10.1; the separate forward and backward kernels took 6.2 + 5.7 and a
+// launch more).  B: a multiple of 8.
+constexpr int kOutRows = 16;
+__global__ void __launch_bounds__(256) out_kernel(const bf16* __restrict__ H3, const float* __restrict__ t,
+                                                  const float* __restrict__ P, const float* __restrict__ Z3, int B,
+                                                  bf16* dZ3, bf16* dZ3t, float* dy, float* loss)
 {
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (b >= B) return;
-    float s = 0.0f;
-    for (int k = lane; k < kW; k += 32) s += __bfloat162float(H3[(size_t)b * kW + k]) * P[ow4 + k];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) y[b] = s + P[ob4];
-}
-
-// L = 1/2 mean (y - t)^2: dy = (y - t)/B, dZ3 = dy w4 gelu'(Z3) (BF16 and its
-// transpose), loss accumulated into *loss.
-__global__ void out_bwd_kernel(const float* __restrict__ y, const float* __restrict__ t,
-                               const float* __restrict__ P, const float* __restrict__ Z3, int B,
-                               bf16* dZ3, bf16* dZ3t, float* dy, float* loss)
-{
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= B * kW) return;
-    const int b = q / kW, k = q % kW;
-    const float r = y[b] - t[b];
-    const float d = r / (float)B;
-    if (k == 0) {
-        dy[b] = d;
-        atomicAdd(loss, 0.5f * r * r / (float)B);
+    __shared__ bf16 tile[kOutRows][kW];
+    const int lane = threadIdx.x & 31, b0 = blockIdx.x * kOutRows;
+    for (int r = threadIdx.x >> 5; r < kOutRows && b0 + r < B; r += 8) {
+        const int b = b0 + r;
+        float s = 0.0f;
+        for (int k = lane; k < kW; k += 32) s += __bfloat162float(H3[(size_t)b * kW + k]) * P[ow4 + k];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const float e = s + P[ob4] - t[b];
+        const float d = e / (float)B;
+        if (lane == 0) {
+            dy[b] = d;
+            atomicAdd(loss, 0.5f * e * e / (float)B);
+        }
+        for (int k = lane; k < kW; k += 32) {
+            const bf16 h = __float2bfloat16(d * P[ow4 + k] * tc::gelu_grad(Z3[(size_t)b * kW + k]));
+            dZ3[(size_t)b * kW + k] = h;
+            tile[r][k] = h;
+        }
     }
-    const bf16 h = __float2bfloat16(d * P[ow4 + k] * tc::gelu_grad(Z3[(size_t)b * kW + k]));
-    dZ3[(size_t)b * kW + k] = h;
-    dZ3t[(size_t)k * B + b] = h;
+    __syncthreads();
+    static_assert(kW == 256);  // a column per thread
+    for (int r = 0; r < kOutRows && b0 + r < B; r += 8) {
+        __align__(16) bf16 h[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) h[i] = tile[r + i][threadIdx.x];
+        *reinterpret_cast<uint4*>(dZ3t + (size_t)threadIdx.x * B + b0 + r) = *reinterpret_cast<const uint4*>(h);
+    }
 }
 
 // Output-layer gradients: g_w4[k] = sum_b dy_b H3[b][k], g_b4 = sum_b dy_b.  A
@@ -401,16 +468,19 @@ __global__ void __launch_bounds__(256) out_wgrad_kernel(const bf16* __restrict__
     }
 }
 
-// Bias gradients from the transposed layer gradient dZt [N x B]: one warp per row.
-__global__ void rowsum_kernel(const bf16* __restrict__ dZt, int N, int B, float* gb)
+// Bias gradients from the transposed layer gradients [kW x B] of the three
+// layers (blockIdx.y): one warp per row.
+__global__ void rowsum_kernel(const bf16* __restrict__ dZ1t, const bf16* __restrict__ dZ2t, const bf16* __restrict__ dZ3t,
+                              int B, float* G)
 {
     const int n = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (n >= N) return;
+    const int lane = threadIdx.x & 31, layer = blockIdx.y;
+    const bf16* dZt = layer == 0 ? dZ1t : (layer == 1 ? dZ2t : dZ3t);
+    if (n >= kW) return;
     float s = 0.0f;
     for (int b = lane; b < B; b += 32) s += __bfloat162float(dZt[(size_t)n * B + b]);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) gb[n] = s;
+    if (lane == 0) G[(layer == 0 ? ob1 : (layer == 1 ? ob2 : ob3)) + n] = s;
 }
 
 __global__ void adam_kernel(float* P, const float* __restrict__ G, float* Mo, float* Vo, int n, float lr,
@@ -584,7 +654,7 @@ amfrw_params params_from(const Family& fam, const double* f, InstanceStore& st)
 struct SgWork {
     bf16 *X = nullptr, *Xt = nullptr, *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *H1t = nullptr, *H2t = nullptr;
     bf16 *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr, *dZ1t = nullptr, *dZ2t = nullptr, *dZ3t = nullptr;
-    float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *y = nullptr, *t = nullptr, *dy = nullptr, *loss = nullptr;
+    float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *t = nullptr, *dy = nullptr, *loss = nullptr;
     int* idx = nullptr;  // training: the epoch's permutation of the rows
     cudaStream_t st = nullptr;
     bool own_stream = false;
@@ -592,7 +662,7 @@ struct SgWork {
     {
         for (void* q : {(void*)X, (void*)Xt, (void*)H1, (void*)H2, (void*)H3, (void*)H1t, (void*)H2t,
                         (void*)dZ1, (void*)dZ2, (void*)dZ3, (void*)dZ1t, (void*)dZ2t, (void*)dZ3t,
-                        (void*)Z1, (void*)Z2, (void*)Z3, (void*)y, (void*)t, (void*)dy, (void*)loss, (void*)idx})
+                        (void*)Z1, (void*)Z2, (void*)Z3, (void*)t, (void*)dy, (void*)loss, (void*)idx})
             cudaFree(q);
         if (own_stream && st) cudaStreamDestroy(st);
         *this = SgWork{};
@@ -651,7 +721,6 @@ int sg_work_alloc(SgWork& w, size_t fwd_rows, size_t train_rows)
     for (bf16** q : {&w.H1t, &w.H2t, &w.dZ1, &w.dZ2, &w.dZ3, &w.dZ1t, &w.dZ2t, &w.dZ3t})
         SG_CUDA(cudaMalloc(q, B2 * train_rows * kW));
     for (float** q : {&w.Z1, &w.Z2, &w.Z3}) SG_CUDA(cudaMalloc(q, F4 * train_rows * kW));
-    SG_CUDA(cudaMalloc(&w.y, F4 * fwd_rows));
     SG_CUDA(cudaMalloc(&w.t, F4 * train_rows));
     SG_CUDA(cudaMalloc(&w.dy, F4 * train_rows));
     SG_CUDA(cudaMalloc(&w.loss, F4));
@@ -718,12 +787,11 @@ int sg_forward(amfrw_surrogate* s, int m, int B, bool train, float* y, const SgW
     if (!rc) rc = tc::gemm(w.H1, kW, s->W2b[m], kW, B, kW, kW, e, st);
     e.bias = s->P[m] + ob3; e.Z = train ? w.Z3 : nullptr; e.H = w.H3; e.Ht = nullptr;
     // a prediction needs the third layer's activations only in its output,
-    // which the product's epilogue forms (out_fwd_kernel's sum in its order)
+    // which the product's epilogue forms (out_kernel's sum in its order)
     e.mode = train ? 1 : 3;
     e.w4 = s->P[m] + ow4;
     e.y = y;
     if (!rc) rc = tc::gemm(w.H2, kW, s->W3b[m], kW, B, kW, kW, e, st);
-    if (!rc && train) out_fwd_kernel<<<cdiv(B * 32, 256), 256, 0, st>>>(w.H3, s->P[m], y, B);
     if (rc) return sg_fail(AMFRW_ECUDA, std::string("surrogate forward: ") + cudaGetErrorString((cudaError_t)rc));
     return AMFRW_OK;
 }
@@ -733,27 +801,22 @@ int sg_backward(amfrw_surrogate* s, int m, int B, const SgWork& w)
 {
     cudaStream_t st = w.st;
     float* G = s->G[m];
-    out_bwd_kernel<<<cdiv(B * kW, 256), 256, 0, st>>>(w.y, w.t, s->P[m], w.Z3, B, w.dZ3, w.dZ3t, w.dy, w.loss);
+    out_kernel<<<cdiv(B, kOutRows), 256, 0, st>>>(w.H3, w.t, s->P[m], w.Z3, B, w.dZ3, w.dZ3t, w.dy, w.loss);
     out_wgrad_kernel<<<kW / 8 + 1, 256, 0, st>>>(w.H3, w.dy, B, G);
     tc::Epi e{};
     e.error = s->err;
     e.ldt = B;
-    // W3, b3
-    e.mode = 0; e.C = G + oW3; e.ldc = kW;
-    int rc = tc::gemm(w.dZ3t, B, w.H2t, B, kW, kW, B, e, st);
-    rowsum_kernel<<<cdiv(kW * 32, 256), 256, 0, st>>>(w.dZ3t, kW, B, G + ob3);
-    // dZ2 = (dZ3 W3) * gelu'(Z2)
+    // dZ2 = (dZ3 W3) * gelu'(Z2), dZ1 = (dZ2 W2) * gelu'(Z1)
     e.mode = 2; e.H = w.dZ2; e.Ht = w.dZ2t; e.Zprev = w.Z2;
-    if (!rc) rc = tc::gemm(w.dZ3, kW, s->W3tb[m], kW, B, kW, kW, e, st);
-    e.mode = 0; e.C = G + oW2; e.ldc = kW;
-    if (!rc) rc = tc::gemm(w.dZ2t, B, w.H1t, B, kW, kW, B, e, st);
-    rowsum_kernel<<<cdiv(kW * 32, 256), 256, 0, st>>>(w.dZ2t, kW, B, G + ob2);
-    // dZ1 = (dZ2 W2) * gelu'(Z1)
-    e.mode = 2; e.H = w.dZ1; e.Ht = w.dZ1t; e.Zprev = w.Z1;
+    int rc = tc::gemm(w.dZ3, kW, s->W3tb[m], kW, B, kW, kW, e, st);
+    e.H = w.dZ1; e.Ht = w.dZ1t; e.Zprev = w.Z1;
     if (!rc) rc = tc::gemm(w.dZ2, kW, s->W2tb[m], kW, B, kW, kW, e, st);
-    e.mode = 0; e.C = G + oW1; e.ldc = kInPad;
-    if (!rc) rc = tc::gemm(w.dZ1t, B, w.Xt, B, kW, kInPad, B, e, st);
-    rowsum_kernel<<<cdiv(kW * 32, 256), 256, 0, st>>>(w.dZ1t, kW, B, G + ob1);
+    // the weight and bias gradients of the three layers
+    const tc::Product wg[3] = {{w.dZ3t, w.H2t, G + oW3, kW, kW, kW},
+                               {w.dZ2t, w.H1t, G + oW2, kW, kW, kW},
+                               {w.dZ1t, w.Xt, G + oW1, kInPad, kW, kInPad}};
+    if (!rc) rc = tc::gemm3(wg, B, B, B, s->err, st);
+    rowsum_kernel<<<dim3(cdiv(kW * 32, 256), 3), 256, 0, st>>>(w.dZ1t, w.dZ2t, w.dZ3t, B, G);
     if (rc) return sg_fail(AMFRW_ECUDA, std::string("surrogate backward: ") + cudaGetErrorString((cudaError_t)rc));
     return AMFRW_OK;
 }
@@ -1091,7 +1154,7 @@ int amfrw_surrogate_fit(amfrw_surrogate* s, const amfrw_params* ps, const double
                 const SgWork& w = tw[(size_t)m];
                 pack_kernel<<<cdiv(B * kInPad, 256), 256, 0, w.st>>>(d_feats, d_targ, w.idx + k * B, 0, B, w.X,
                                                                     w.Xt, w.t);
-                rc = sg_forward(s, m, B, true, w.y, w);
+                rc = sg_forward(s, m, B, true, nullptr, w);
                 if (rc == AMFRW_OK) rc = sg_backward(s, m, B, w);
                 adam_kernel<<<cdiv(kParams, 256), 256, 0, w.st>>>(s->P[m], s->G[m], s->Mo[m], s->Vo[m], kParams,
                                                                  lr_t, 0.9f, 0.999f, 1e-8f, bc1, bc2);
@@ -1318,7 +1381,7 @@ int amfrw_surrogate_grad(amfrw_surrogate* s, int32_t member, const float* x_norm
     cudaMemsetAsync(s->w.loss, 0, sizeof(float), st);
     cudaMemsetAsync(s->G[member], 0, sizeof(float) * kParams, st);
     pack_kernel<<<cdiv(rows * kInPad, 256), 256, 0, st>>>(d_x, d_t, nullptr, 0, rows, s->w.X, s->w.Xt, s->w.t);
-    int rc = sg_forward(s, member, rows, true, s->w.y, s->w);
+    int rc = sg_forward(s, member, rows, true, nullptr, s->w);
     if (rc == AMFRW_OK) rc = sg_backward(s, member, rows, s->w);
     if (rc == AMFRW_OK) {
         cudaMemcpyAsync(grad_out, s->G[member], sizeof(float) * kParams, cudaMemcpyDeviceToHost, st);

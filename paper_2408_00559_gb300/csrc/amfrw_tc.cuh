@@ -161,7 +161,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
 // elements of K, then the mbarriers (full and empty per stage, done) and the
 // TMEM address.  A stage's operand is one box of rows x 128 bytes.  (1 KB more
 // than needed, to start on a 1024-byte boundary.)
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 8;
 constexpr int kTurnBytes = 32 * 144;  // a warp's buffer in the epilogue
 constexpr int kTileA = kBM * kBK * 2;
 __host__ __device__ constexpr int stage_bytes(int BN) { return kTileA + BN * kBK * 2; }
@@ -211,10 +211,9 @@ __device__ __forceinline__ float gelu_grad(float z)
     return cdf + z * pdf;
 }
 
-// C-tile = A[m0:m0+128, :] * B[n0:n0+BN, :]^T; grid (M/128, N/BN).
-__global__ void __launch_bounds__(kThreads, 2)
-    gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M,
-                     int N, int K, int BN, int S, Epi epi)
+// C-tile = A[m0:m0+128, :] * B[n0:n0+BN, :]^T on one block.
+__device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensorMap& tmB, int m0, int n0, int M, int N,
+                                          int K, int BN, int S, const Epi& epi)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -224,8 +223,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     __shared__ int s_fail;
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
-    const int m0 = blockIdx.x * kBM;
-    const int n0 = blockIdx.y * BN;
     const uint32_t ncols = BN <= 32 ? 32u : (BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u));
     auto full = [&](int st) { return smem_u32(bars + st); };
     auto empty = [&](int st) { return smem_u32(bars + kMaxStages + st); };
@@ -250,15 +247,14 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (tid == 0) {
         const uint32_t idesc = instr_desc_bf16(kBM, BN);
         const uint32_t tx = (uint32_t)SB;
-        int pend[kMaxStages];  // loads issued and not yet waited for: their chunk, or -1
+        int issued = 0, waited = 0;  // chunks: loads issued, loads waited for
         auto load = [&](int i, int st) {
             const uint32_t a = smem_u32(smem + st * SB), b = a + kTileA;
             mbar_expect_tx(full(st), tx);
             tma_load_2d(a, &tmA, i * kBK, m0, full(st));
             tma_load_2d(b, &tmB, i * kBK, n0, full(st));
-            pend[st] = i;
+            issued = i + 1;
         };
-        for (int st = 0; st < kMaxStages; ++st) pend[st] = -1;
         for (int i = 0; i < S && i < nk; ++i) load(i, i);
         bool ok = true;
         for (int i = 0; i < nk && ok; ++i) {
@@ -266,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             const uint32_t ph = (uint32_t)((i / S) & 1);
             ok = mbar_wait(full(st), ph);
             if (!ok) break;
-            pend[st] = -1;
+            waited = i + 1;
             fence_after();
             const int kc = (K - i * kBK) < kBK ? (K - i * kBK) : kBK;  // multiple of 16
             const uint32_t a = smem_u32(smem + st * SB), b = a + kTileA;
@@ -288,8 +284,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (!ok) {
             // wait (bounded) for the loads still in flight, so that none lands
             // in shared memory after the block has gone
-            for (int st = 0; st < S; ++st)
-                if (pend[st] >= 0) mbar_wait(full(st), (uint32_t)((pend[st] / S) & 1));
+            for (int c = waited; c < issued; ++c) mbar_wait(full(c % S), (uint32_t)((c / S) & 1));
             s_fail = 1;
         }
     }
@@ -445,6 +440,37 @@ __global__ void __launch_bounds__(kThreads, 2)
     fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, ncols);
+}
+
+// One product; grid (M/128, N/BN).
+__global__ void __launch_bounds__(kThreads, 2)
+    gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M,
+                     int N, int K, int BN, int S, const __grid_constant__ Epi epi)
+{
+    gemm_tile(tmA, tmB, blockIdx.x * kBM, blockIdx.y * BN, M, N, K, BN, S, epi);
+}
+
+// Up to three products of one K into FP32 results in one launch, a block per
+// tile: the weight gradients of a training batch, none of which has tiles for
+// more than a tenth of the SMs.
+struct Jobs {
+    CUtensorMap a[3], b[3];
+    float* C[3];
+    int ldc[3], M[3], N[3], BN[3];
+    int first[4];  // the product's first block
+    int K, S;
+    int* error;
+};
+__global__ void __launch_bounds__(kThreads, 2) gemm_bf16_batch_kernel(const __grid_constant__ Jobs j)
+{
+    const int q = (int)blockIdx.x < j.first[1] ? 0 : ((int)blockIdx.x < j.first[2] ? 1 : 2);
+    const int t = blockIdx.x - j.first[q], rt = (j.M[q] + kBM - 1) / kBM;
+    Epi e{};
+    e.mode = 0;
+    e.C = j.C[q];
+    e.ldc = j.ldc[q];
+    e.error = j.error;
+    gemm_tile(j.a[q], j.b[q], t % rt * kBM, t / rt * j.BN[q], j.M[q], j.N[q], j.K, j.BN[q], j.S, e);
 }
 
 }  // namespace tc
