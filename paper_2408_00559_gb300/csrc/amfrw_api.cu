@@ -366,8 +366,10 @@ struct Plan {
     int glog_delta = 0;     // warp groups: lanes per grid widened by 2^glog_delta (autotuned)
     bool lean = false;      // no spare global scratch (plan_host)
     // streams and events that let a solve's launches overlap (none: one after
-    // the other)
-    static constexpr int kSides = 4;
+    // the other).  Two at most: each costs a plan 50 us, and more launches than
+    // three at a time measured no faster.
+    static constexpr int kSides = 2;
+    int sides = 0;
     cudaStream_t side[kSides] = {};
     cudaEvent_t fork = nullptr, join[kSides] = {};
     bool shared_u = false;  // d_u belongs to another plan (the FP64 re-solve writes there)
@@ -945,7 +947,8 @@ int build_plan(const amfrw_params* ps, int n, void* stream, bool keep_state, boo
                              cudaMemcpyHostToDevice, P.stream));
     CUDA_TRY(cudaMemsetAsync(P.d_u, 0, sizeof(double) * P.coefs.size(), P.stream));
     if (overlap && launch_records(P).size() > 1) {
-        for (int q = 0; q < Plan::kSides; ++q) {
+        P.sides = std::min((int)launch_records(P).size() - 1, Plan::kSides);
+        for (int q = 0; q < P.sides; ++q) {
             CUDA_TRY(cudaStreamCreateWithFlags(&P.side[q], cudaStreamNonBlocking));
             CUDA_TRY(cudaEventCreateWithFlags(&P.join[q], cudaEventDisableTiming));
         }
@@ -1105,7 +1108,7 @@ int run_solve(Plan& P, int steps, int flags, cudaEvent_t* ev = nullptr)
     if (ev) CUDA_TRY(cudaStreamIsCapturing(P.stream, &cap));
     const unsigned rec_flags = cap == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault;
     const bool overlap = !ev && P.fork && recs.size() > 1;
-    const int used = overlap ? std::min<int>((int)recs.size() - 1, Plan::kSides) : 0;
+    const int used = overlap ? std::min<int>((int)recs.size() - 1, P.sides) : 0;
     if (overlap) {
         CUDA_TRY(cudaEventRecord(P.fork, P.stream));
         for (int q = 0; q < used; ++q) CUDA_TRY(cudaStreamWaitEvent(P.side[q], P.fork, 0));

@@ -17,18 +17,20 @@
 //
 // Mixed precision: the same operations in the same order as the warp groups'
 // solve_item_mixed, so that a price does not depend on which of the two a
-// grid went through.  Bound by instruction issue (48 % of the issue slots, 16
+// grid went through.  Bound by instruction issue (43 % of the issue slots, 16
 // warps per SM; what it waits for is shared-memory latency and the group's
 // barriers).  FP64: the pipe is the bound (one warp instruction per 16 cycles
 // and SM), so the stencil is kept in the form with the fewest FP64
-// instructions (neighbour sums with one centre coefficient, a term per
-// neighbour that exists) and a line is eliminated by one thread (3
-// instructions a row, against 2 log2 P + 3 of a line shared by P lanes).
+// instructions that does not cancel on long axes (second differences 2 (X+ - X)
+// - (X+ - X-), the gradient shared with the cross terms; neighbour sums with a
+// centre coefficient on axes of one and two rows; a term per neighbour that
+// exists) and a line is eliminated by one thread (3 instructions a row, against
+// 2 log2 P + 3 of a line shared by P lanes).
 //
 // Measured, the warp groups first: 1024 d=4 level-5 instances in FP64 34.7 ->
-// 18.9 ms; the uneven book of 256 (N = 4, 6, 8) in mixed precision 31.4 ->
-// 18.7 ms; 512 d=6 level-6 instances in mixed precision, host to host, 88.4 ->
-// 49.3 ms; 64 d=6 level-5 instances in FP64 17.5 -> 5.7 ms.
+// 20.2 ms; the uneven book of 256 (N = 4, 6, 8) in mixed precision 31.4 ->
+// 17.4 ms; 512 d=6 level-6 instances in mixed precision, host to host, 88.4 ->
+// 49.1 ms; 64 d=6 level-5 instances in FP64 17.5 -> 5.7 ms.
 #pragma once
 #include "amfrw_solver.cuh"
 
