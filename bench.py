@@ -79,11 +79,14 @@ CALIB_Q = 0.999
 CALIB_N = 16384
 
 # DRAM bytes (read + write) of the solver launches of one 256-instance batched
-# mixed-precision batch in its multi-class configuration (one launch per N):
-# one ncu capture, dram__bytes_read.sum 804 096 + 5 778 176 + 13 012 480 and
-# dram__bytes_write.sum 0 + 292 864 + 276 690 432 for N = 4, 6, 8 (the writes:
-# local-memory stack frames of the per-grid setup calls written back from L2).
-C4_DRAM_BYTES_PER_BATCH = 804096 + 5778176 + 13012480 + 292864 + 276690432
+# mixed-precision batch (bundles of N = 8 and 6, warp groups of N = 8, 6, 4):
+# one ncu capture, dram__bytes_read.sum 23 177 472 + 16 993 280 + 5 324 288 +
+# 3 241 472 + 597 504 and dram__bytes_write.sum 119 200 768 + 3 458 816 +
+# 14 230 784 + 25 856 + 0 (the writes: line-solve factors of the largest bundles
+# and local-memory stack frames of the per-grid setup, written back from L2).
+C4_DRAM_LAUNCHES = 5
+C4_DRAM_BYTES_PER_BATCH = (23177472 + 16993280 + 5324288 + 3241472 + 597504
+                           + 119200768 + 3458816 + 14230784 + 25856)
 
 
 def parse():
@@ -517,7 +520,7 @@ def roofline_entry(insts, kernel_ms, peak64, peak32, mixed):
     t64 = f64 / (peak64 * 1e12)
     pipe = "fp32" if t32 >= t64 else "fp64"
     ops, peak = (f32, peak32) if pipe == "fp32" else (f64, peak64)
-    return {"bound": "alu", "pipe": pipe, "kernel": "solve_kernel (all solver launches of a batch)",
+    return {"bound": "alu", "pipe": pipe, "kernel": "bundle_kernel and solve_kernel (all solver launches of a batch)",
             "achieved": ops / t / 1e12, "peak": peak, "unit": "TFLOP/s", "frac": max(t32, t64) / t,
             "traffic": None,
             "kernel_ms_per_batch": kernel_ms, "fp32_ops_per_batch": f32, "fp64_ops_per_batch": f64,
@@ -596,10 +599,10 @@ def run_ours(args, rank, world, local_rank):
     roof["solver_launches_per_batch"] = launches_per_batch
     roof["launch_ms"] = [{"N": int(kt[0]), "ms": round(float(np.mean([k[q][1] for k in ktimes])), 3)}
                          for q, kt in enumerate(ktimes[0])]
-    if name == "c4" and B == 256 and launches_per_batch == 3 and not args.global_grids:
+    if name == "c4" and B == 256 and launches_per_batch == C4_DRAM_LAUNCHES and not args.global_grids:
         roof["traffic"] = C4_DRAM_BYTES_PER_BATCH
-        roof["traffic_note"] = ("DRAM bytes of the batch's three solver launches, one ncu capture: "
-                                "parameter records, grid list, values, local-memory write-back")
+        roof["traffic_note"] = ("DRAM bytes of the batch's solver launches, one ncu capture: "
+                                "parameter records, grid list, values, factor scratch, local-memory write-back")
 
     # accuracy: mixed prices against the FP64 GPU prices of the same instances
     # (the FP64 path is pinned to the oracle at 1e-12 by the parity tests),
