@@ -59,6 +59,9 @@ __global__ void __launch_bounds__(KIND == kWarpGroup ? 128 : kCtaMaxThreads, KIN
                 if (csize > 1) cg::this_cluster().sync();
                 else __syncthreads();
             };
+            // another block's shared memory may be written only once that
+            // block has started (the barriers below order the later passes)
+            if (csize > 1) csync();
             for (;;) {
                 if (crank == 0 && threadIdx.x == 0) {
                     const int v = atomicAdd(a.queue, 1);
