@@ -449,12 +449,17 @@ __device__ void solve_item_f64(const SolveArgs& a, const Item& it, unsigned char
         }
         csync();
     };
-    // the stage's solves, `from` into `to`
+    // the stage's solves, `from` into `to`.  Lines along the split axis read the
+    // owners' copies of a vector in shared memory; right-hand sides that found
+    // no room there (four vectors of 8192 nodes do not fit) lie in the
+    // cluster's one slice and are read directly: only a shared address may be
+    // mapped to another block.
+    const bool k0_fast = (y.fast & 8) != 0;
     auto solves = [&](const double* from, double* to) {
         const double* src = from;
         for (int ax = 0; ax < N; ++ax) {
             if ((s.skip >> ax) & 1) continue;
-            const bool far = remote && ax == sl.x;
+            const bool far = remote && ax == sl.x && (src != K0 || k0_fast);
             sweep_f64<N>(
                 s, ax, lu + lu_at(ax), to, sl, ax == 0 && own0 ? crank * (s.M[N - 1] >> sl.c) : 0, tid, nt,
                 [&](int t, int J) -> double {
