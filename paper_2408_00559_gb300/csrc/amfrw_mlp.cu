@@ -87,9 +87,6 @@ int tile_stages(int BN, int nk, int tiles, int sms)
     return S;
 }
 
-// (the epilogue turns its values through the stages' memory)
-int tile_smem(int BN, int S) { return std::max(smem_bytes(BN, S), 1024 + kThreads / 32 * kTurnBytes); }
-
 // Raises the kernels' dynamic shared-memory limit, an attribute per device,
 // once on every device that launches them (to the most any launch asks for).
 int raise_limits(int dev)
@@ -124,7 +121,7 @@ int gemm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M
     if (const int rc = raise_limits(dev)) return rc;
     CUtensorMap tA, tB;
     if (!make_map(&tA, A, M, K, lda, kBM) || !make_map(&tB, B, N, K, ldb, BN)) return (int)cudaErrorInvalidValue;
-    gemm_bf16_kernel<<<grid, kThreads, tile_smem(BN, S), st>>>(tA, tB, M, N, K, BN, S, epi);
+    gemm_bf16_kernel<<<grid, kThreads, smem_bytes(BN, S), st>>>(tA, tB, M, N, K, BN, S, epi);
     return (int)cudaGetLastError();
 }
 
@@ -159,7 +156,7 @@ int gemm3(const Product (&p)[3], int lda, int ldb, int K, int* error, cudaStream
     }
     j.S = tile_stages(wide, (K + kBK - 1) / kBK, j.first[3], sms);
     if (const int rc = raise_limits(dev)) return rc;
-    gemm_bf16_batch_kernel<<<j.first[3], kThreads, tile_smem(wide, j.S), st>>>(j);
+    gemm_bf16_batch_kernel<<<j.first[3], kThreads, smem_bytes(wide, j.S), st>>>(j);
     return (int)cudaGetLastError();
 }
 

@@ -158,14 +158,20 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
 }
 
 // Shared memory of one CTA: S stages of A (128 rows) and B (BN rows) x 64
-// elements of K, then the mbarriers (full and empty per stage, done) and the
-// TMEM address.  A stage's operand is one box of rows x 128 bytes.  (1 KB more
-// than needed, to start on a 1024-byte boundary.)
+// elements of K, which the epilogue's buffers reuse, then, behind both, the
+// mbarriers (full and empty per stage, done) and the TMEM address.  A stage's
+// operand is one box of rows x 128 bytes.  (1 KB more than needed, to start on
+// a 1024-byte boundary.)
 constexpr int kMaxStages = 8;
 constexpr int kTurnBytes = 32 * 144;  // a warp's buffer in the epilogue
 constexpr int kTileA = kBM * kBK * 2;
 __host__ __device__ constexpr int stage_bytes(int BN) { return kTileA + BN * kBK * 2; }
-__host__ __device__ constexpr int smem_bytes(int BN, int stages) { return 1024 + stages * stage_bytes(BN) + 8 * (2 * kMaxStages + 1) + 16; }
+__host__ __device__ constexpr int bars_offset(int BN, int stages)
+{
+    const int st = stages * stage_bytes(BN), turn = kThreads / 32 * kTurnBytes;
+    return st > turn ? st : turn;
+}
+__host__ __device__ constexpr int smem_bytes(int BN, int stages) { return 1024 + bars_offset(BN, stages) + 8 * (2 * kMaxStages + 1) + 16; }
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t addr, uint32_t bytes)
 {
@@ -218,8 +224,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int SB = stage_bytes(BN);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * SB);  // full[kMaxStages], empty[kMaxStages], done
-    uint32_t* taddr_slot = reinterpret_cast<uint32_t*>(smem + S * SB + 8 * (2 * kMaxStages + 1));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bars_offset(BN, S));  // full[kMaxStages], empty[kMaxStages], done
+    uint32_t* taddr_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 1);
     __shared__ int s_fail;
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -269,7 +275,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
             for (int kk = 0; kk < kc / 16; ++kk) {
                 mma_bf16(tmem, smem_desc(a + kk * 32), smem_desc(b + kk * 32), idesc, (i > 0 || kk > 0) ? 1u : 0u);
             }
-            mma_commit(empty(st));
+            if (i + S < nk) mma_commit(empty(st));  // (only what a refill waits for)
             // refill the previous chunk's stage once its MMAs are done (the
             // current chunk's MMAs keep the tensor pipe busy meanwhile)
             const int prev = i - 1, next = prev + S;
@@ -297,7 +303,8 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
         if (tid == 0) atomicExch(epi.error, 1);
     } else {
         // epilogue: lane = row m0 + 32 warp + lane, 32 columns at a time.  The
-        // stages are free now (their loads and MMAs are done): each warp
+        // stages are free now (their loads and MMAs are done; the mbarriers,
+        // where an arrive may still land, lie behind them): each warp
         // turns its 32 x 32 values there, rows 144 bytes apart (FP32) or 80
         // (BF16), so that both the row-wise and the line-wise 16-byte
         // accesses are free of bank conflicts.
