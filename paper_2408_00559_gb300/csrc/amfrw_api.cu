@@ -1239,9 +1239,11 @@ namespace {
 std::mutex g_tune_mutex;
 std::map<std::string, int> g_tune_cache;
 
+// (The signature starts with the version of the kernels and of the tuner: a
+// choice kept in a file by another build may be of launches that are gone.)
 std::string class_signature(const Plan& P)
 {
-    std::string sig;
+    std::string sig = "2|";
     for (const LaunchClass& c : P.classes) {
         sig += std::to_string(c.N) + (c.mixed ? "m" : "d") + (c.kind == kWarpGroup ? "w" : (c.kind == kCtaGroup ? "c" : "g")) +
                std::to_string(P.items[c.item_begin].L) + ":" +
@@ -1610,14 +1612,17 @@ int amfrw_batch_autotune(amfrw_batch* b, int32_t trials, int32_t* use_multi_out)
     const int steps = P.insts[0].n_steps;
     const std::string sig = class_signature(P);  // of the plan as built, before any move
     const std::vector<LaunchClass> base = P.classes;
-    // time `trials` solves (after a warm-up); per-record times if rec != nullptr
-    auto timed = [&](float& total, std::vector<float>* rec) -> int {
-        const size_t nrec = launch_records(P).size();
+    // time `trials` solves (after a warm-up); the times of each class's own
+    // launch if by_class != nullptr (by class: a launch's place among the
+    // solve's launches depends on its kind, which step 3 changes)
+    auto timed = [&](float& total, std::vector<float>* by_class) -> int {
+        const std::vector<LaunchRec> recs = launch_records(P);
+        const size_t nrec = recs.size();
         std::vector<cudaEvent_t> ev(2 * nrec, nullptr);
         for (cudaEvent_t& e : ev) CUDA_TRY(cudaEventCreate(&e));
         int st = run_solve(P, steps, 0);
         total = 0.f;
-        if (rec) rec->assign(nrec, 0.f);
+        if (by_class) by_class->assign(P.classes.size(), 0.f);
         for (int k = 0; k < trials && st == AMFRW_OK; ++k) {
             st = run_solve(P, steps, 0, ev.data());
             if (st == AMFRW_OK && cudaEventSynchronize(ev.back()) != cudaSuccess) st = fail(AMFRW_ECUDA, "timing");
@@ -1625,7 +1630,7 @@ int amfrw_batch_autotune(amfrw_batch* b, int32_t trials, int32_t* use_multi_out)
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, ev[2 * r], ev[2 * r + 1]);
                 total += ms;
-                if (rec) (*rec)[r] += ms;
+                if (by_class && recs[r].cls >= 0) (*by_class)[(size_t)recs[r].cls] += ms;
             }
         }
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
@@ -1682,25 +1687,17 @@ int amfrw_batch_autotune(amfrw_batch* b, int32_t trials, int32_t* use_multi_out)
     for (size_t c = 0; c < P.classes.size(); ++c)
         if (P.classes[c].kind == kCtaGroup) cta.push_back((int)c);
     if (!cta.empty()) {
-        // launch record of each CTA class
-        std::vector<size_t> at;
-        {
-            const std::vector<LaunchRec> recs = launch_records(P);
-            for (int c : cta)
-                for (size_t r = 0; r < recs.size(); ++r)
-                    if (recs[r].cls == c) at.push_back(r);
-        }
         float tot[2];
-        std::vector<float> rec[2];
-        st = timed(tot[0], &rec[0]);
+        std::vector<float> ms[2];  // by class
+        st = timed(tot[0], &ms[0]);
         for (int c : cta)
             if (st == AMFRW_OK) st = class_to_global(P, c);
         if (st == AMFRW_OK) st = relayout_scratch(P);
-        if (st == AMFRW_OK) st = timed(tot[1], &rec[1]);
+        if (st == AMFRW_OK) st = timed(tot[1], &ms[1]);
         if (st != AMFRW_OK) return st;
         P.classes = base;  // back to shared memory, then move the classes that were faster
         for (size_t k = 0; k < cta.size(); ++k) {
-            if (rec[1][at[k]] < rec[0][at[k]]) {
+            if (ms[1][(size_t)cta[k]] < ms[0][(size_t)cta[k]]) {
                 choice |= 1 << (1 + (int)k);
                 st = class_to_global(P, cta[k]);
                 if (st != AMFRW_OK) return st;
