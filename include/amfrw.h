@@ -218,8 +218,9 @@ int amfrw_batch_launches(const amfrw_batch *b, int32_t *n_launches);
  * batches: up to 32 instances of one grid together), one persistent
  * multi-class launch per (N, precision) for the other grids of that size (when
  * that strategy is selected), and one launch per remaining (N, precision,
- * grid class).  amfrw_batch_kernel_times synchronises and writes, for the
- * last run, the device milliseconds of each solver launch to
+ * grid class).  With timing on the launches run one after the
+ * other; without, they overlap.  amfrw_batch_kernel_times synchronises and
+ * writes, for the last run, the device milliseconds of each solver launch to
  * ms_out[0..*n_out-1] (at most cap entries), the Inner-node-steps it advanced
  * (sum over its grids of Inner nodes x steps) to node_steps_out (may be NULL)
  * and its N to dims_out (may be NULL). */
@@ -230,13 +231,15 @@ int amfrw_batch_kernel_times(amfrw_batch *b, float *ms_out, double *node_steps_o
 /* Autotuning of the launch strategy, of the warp groups' width and of where
  * grid states live (the paper has no counterpart; its CPU code schedules
  * grids with OpenMP's dynamic schedule).  Times, on this batch and device
- * (`trials` solves each after a warm-up): (1) per-class launches against one
+ * (`trials` solves each after a warm-up, their launches overlapping as a
+ * batch's do): (1) per-class launches against one
  * persistent multi-class launch for the warp-solved grids; (2) the warp
  * groups' width: each grid on its natural number of lanes (two nodes per
  * lane) against twice as many (one node per lane, one more level of parallel
  * cyclic reduction and fewer Thomas rows per line); (3) for every CTA class
  * (grids in shared memory) its launch with the grid states in shared memory
- * against in global memory, class by class.  Keeps the faster choices (the
+ * against in global memory, class by class (here one launch after the other).
+ * Keeps the faster choices (the
  * single persistent launch unless the per-class launches are more than 10 %
  * faster) and caches them in-process under the batch's class signature (and, if the
  * environment variable AMFRW_TUNE_CACHE names a file, appends them there),

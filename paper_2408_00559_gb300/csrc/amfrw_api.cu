@@ -1612,21 +1612,25 @@ int amfrw_batch_autotune(amfrw_batch* b, int32_t trials, int32_t* use_multi_out)
     const int steps = P.insts[0].n_steps;
     const std::string sig = class_signature(P);  // of the plan as built, before any move
     const std::vector<LaunchClass> base = P.classes;
-    // time `trials` solves (after a warm-up); the times of each class's own
-    // launch if by_class != nullptr (by class: a launch's place among the
-    // solve's launches depends on its kind, which step 3 changes)
+    // time `trials` solves (after a warm-up) as a batch runs them, their
+    // launches overlapping; or, if by_class != nullptr, one launch after the
+    // other, with the times of each class's own launch (by class: a launch's
+    // place among the solve's launches depends on its kind, which step 3
+    // changes)
     auto timed = [&](float& total, std::vector<float>* by_class) -> int {
         const std::vector<LaunchRec> recs = launch_records(P);
-        const size_t nrec = recs.size();
-        std::vector<cudaEvent_t> ev(2 * nrec, nullptr);
+        const size_t nev = by_class ? 2 * recs.size() : 2;
+        std::vector<cudaEvent_t> ev(nev, nullptr);
         for (cudaEvent_t& e : ev) CUDA_TRY(cudaEventCreate(&e));
         int st = run_solve(P, steps, 0);
         total = 0.f;
         if (by_class) by_class->assign(P.classes.size(), 0.f);
         for (int k = 0; k < trials && st == AMFRW_OK; ++k) {
-            st = run_solve(P, steps, 0, ev.data());
+            if (!by_class && cudaEventRecord(ev[0], P.stream) != cudaSuccess) st = fail(AMFRW_ECUDA, "timing");
+            if (st == AMFRW_OK) st = run_solve(P, steps, 0, by_class ? ev.data() : nullptr);
+            if (st == AMFRW_OK && !by_class && cudaEventRecord(ev[1], P.stream) != cudaSuccess) st = fail(AMFRW_ECUDA, "timing");
             if (st == AMFRW_OK && cudaEventSynchronize(ev.back()) != cudaSuccess) st = fail(AMFRW_ECUDA, "timing");
-            for (size_t r = 0; r < nrec && st == AMFRW_OK; ++r) {
+            for (size_t r = 0; 2 * r < nev && st == AMFRW_OK; ++r) {
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, ev[2 * r], ev[2 * r + 1]);
                 total += ms;
