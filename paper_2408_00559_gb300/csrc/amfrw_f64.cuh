@@ -54,12 +54,16 @@ struct Slab {
 // streams its R rows B at a time: an FP64 instruction's result is some tens of
 // cycles away and a store waits for it, so the rows of a batch are loaded
 // first, computed side by side, and stored last; elimination, the one chain,
-// takes a single multiply-add per row each way.
-template <int N, int B, class Get, class Put>
+// takes a single multiply-add per row each way.  MANY: there are several
+// batches, and a batch's rows and factors are loaded while the one before it
+// is computed (a line of 16384 rows in global scratch waited for its factors at
+// every batch: 4.8 ms a step, 2.8 so; one of 4096 in shared memory, whose
+// factors do not fit there, 0.79, 0.64).  Otherwise B = R.
+template <int N, int B, bool MANY, class Get, class Put>
 __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, const double* lu, double* dst, const Slab& sl,
                                                int cls0, int tid, int nt, Get get, Put put)
 {
-    const int M = s.M[axis], plog = s.plog[axis], P = 1 << plog, R = M >> plog, S = s.luS[axis];
+    const int M = s.M[axis], plog = s.plog[axis], P = 1 << plog, R = MANY ? M >> plog : B, S = s.luS[axis];
     const int lvA = s.lv[axis], sh = s.sh[axis], Spa = s.Sp[axis];
     const bool cut = axis == sl.x;  // lines through all slabs: shared out
     const int nl = (s.L >> lvA) >> sl.c;
@@ -82,6 +86,15 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
         const int st = P << sh, tp = t0 + (p << sh);
         bool first = true;
         auto in = [&](int q) -> double { return first ? get(tp + q * st, J0 + q * PSp) : dst[J0 + q * PSp]; };
+        // factor e of the batch of rows from q on
+        auto factors = [&](double (&f)[B], bool on, int q, int e) {
+#pragma unroll
+            for (int i = 0; i < B; ++i) f[i] = on ? tb[(q + i) * PS + e] : 0.0;
+        };
+        auto rows = [&](double (&v)[B], bool on, int q) {
+#pragma unroll
+            for (int i = 0; i < B; ++i) v[i] = on ? in(q + i) : 0.0;
+        };
         double x[B];
 #pragma unroll 1
         for (int k = 0; k < plog; ++k) {
@@ -89,73 +102,102 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
             const int sm = (p - d) & (P - 1), sp = (p + d) & (P - 1);
             const bool send_prev = p >= P - d, send_next = p < d;
             double prev = 0.0;  // the row before the batch, as it was
-#pragma unroll
-            for (int i = 0; i < B; ++i) x[i] = act ? in(i) : 0.0;
+            double al[B], ga[B];
+            rows(x, act, 0);
+            factors(al, act, 0, 2 * k);
+            factors(ga, act, 0, 2 * k + 1);
 #pragma unroll 1
             for (int q0 = 0; q0 < R; q0 += B) {
-                const bool more = act && q0 + B < R;
-                double nx[B], v[B];
-#pragma unroll
-                for (int i = 0; i < B; ++i) nx[i] = more ? in(q0 + B + i) : 0.0;
+                double nx[B], na[B], ng[B], v[B];
+                nx[0] = 0.0;
+                if constexpr (MANY) {
+                    const bool more = act && q0 + B < R;
+                    rows(nx, more, q0 + B);
+                    factors(na, more, q0 + B, 2 * k);
+                    factors(ng, more, q0 + B, 2 * k + 1);
+                }
 #pragma unroll
                 for (int i = 0; i < B; ++i) {
                     const double vm = shfl(send_prev ? (i > 0 ? x[i > 0 ? i - 1 : 0] : prev) : x[i], sm, P, 0xffffffffu);
                     const double vp = shfl(send_next ? (i < B - 1 ? x[i < B - 1 ? i + 1 : i] : nx[0]) : x[i], sp, P, 0xffffffffu);
-                    const double* row = tb + (q0 + i) * PS + 2 * k;
-                    const double al = act ? row[0] : 0.0, ga = act ? row[1] : 0.0;
-                    v[i] = fma(-ga, vp, fma(-al, vm, x[i]));
+                    v[i] = fma(-ga[i], vp, fma(-al[i], vm, x[i]));
                 }
                 prev = x[B - 1];
                 if (act) {
 #pragma unroll
                     for (int i = 0; i < B; ++i) dst[J0 + (q0 + i) * PSp] = v[i];
                 }
+                if constexpr (MANY) {
 #pragma unroll
-                for (int i = 0; i < B; ++i) x[i] = nx[i];
+                    for (int i = 0; i < B; ++i) {
+                        x[i] = nx[i];
+                        al[i] = na[i];
+                        ga[i] = ng[i];
+                    }
+                }
             }
             first = false;
         }
         if (act) {
-            const double* th = tb + 2 * plog;
-            double y = 0.0;
-#pragma unroll
-            for (int i = 0; i < B; ++i) x[i] = in(i);
+            const int e = 2 * plog;
+            double y = 0.0, lo[B], iv[B];
+            rows(x, true, 0);
+            factors(lo, true, 0, e);
+            factors(iv, true, 0, e + 1);
 #pragma unroll 1
             for (int q0 = 0; q0 < R; q0 += B) {
-                double nx[B];
-                const bool more = q0 + B < R;
+                double nx[B], nlo[B], niv[B];
+                const bool more = MANY && q0 + B < R;
+                if constexpr (MANY) {
+                    rows(nx, more, q0 + B);
+                    factors(nlo, more, q0 + B, e);
+                    factors(niv, more, q0 + B, e + 1);
+                }
 #pragma unroll
-                for (int i = 0; i < B; ++i) nx[i] = more ? in(q0 + B + i) : 0.0;
-#pragma unroll
-                for (int i = 0; i < B; ++i) x[i] *= th[(q0 + i) * PS + 1];
+                for (int i = 0; i < B; ++i) x[i] *= iv[i];
 #pragma unroll
                 for (int i = 0; i < B; ++i) {
-                    if (i > 0 || q0 > 0) x[i] = fma(-th[(q0 + i) * PS], y, x[i]);
+                    if (i > 0 || q0 > 0) x[i] = fma(-lo[i], y, x[i]);
                     y = x[i];
                 }
-                if (more) {
+                if constexpr (MANY) {
+                    if (more) {
 #pragma unroll
-                    for (int i = 0; i < B; ++i) dst[J0 + (q0 + i) * PSp] = x[i];
+                        for (int i = 0; i < B; ++i) dst[J0 + (q0 + i) * PSp] = x[i];
 #pragma unroll
-                    for (int i = 0; i < B; ++i) x[i] = nx[i];
+                        for (int i = 0; i < B; ++i) {
+                            x[i] = nx[i];
+                            lo[i] = nlo[i];
+                            iv[i] = niv[i];
+                        }
+                    }
                 }
             }
             // back from the last batch, which is still in x
+            double up[B];
+            factors(up, true, R - B, e + 2);
+            first = false;
 #pragma unroll 1
             for (int q0 = R - B; q0 >= 0; q0 -= B) {
-                double nx[B];
-                const bool more = q0 > 0;
-#pragma unroll
-                for (int i = 0; i < B; ++i) nx[i] = more ? dst[J0 + (q0 - B + i) * PSp] : 0.0;
+                double nx[B], nup[B];
+                if constexpr (MANY) {
+                    rows(nx, q0 > 0, q0 - B);
+                    factors(nup, q0 > 0, q0 - B, e + 2);
+                }
 #pragma unroll
                 for (int i = B - 1; i >= 0; --i) {
-                    if (i < B - 1 || q0 + B < R) x[i] = fma(-th[(q0 + i) * PS + 2], y, x[i]);
+                    if (i < B - 1 || q0 + B < R) x[i] = fma(-up[i], y, x[i]);
                     y = x[i];
                 }
 #pragma unroll
                 for (int i = 0; i < B; ++i) put(tp + (q0 + i) * st, J0 + (q0 + i) * PSp, x[i]);
+                if constexpr (MANY) {
 #pragma unroll
-                for (int i = 0; i < B; ++i) x[i] = nx[i];
+                    for (int i = 0; i < B; ++i) {
+                        x[i] = nx[i];
+                        up[i] = nup[i];
+                    }
+                }
             }
         }
     }
@@ -166,9 +208,10 @@ __device__ __forceinline__ void sweep_f64(const Shape<N>& s, int axis, const dou
                                           int cls0, int tid, int nt, Get get, Put put)
 {
     const int R = s.M[axis] >> s.plog[axis];
-    if (R >= 4) sweep_f64_rows<N, 4>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
-    else if (R == 2) sweep_f64_rows<N, 2>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
-    else sweep_f64_rows<N, 1>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    if (R > 4) sweep_f64_rows<N, 4, true>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else if (R == 4) sweep_f64_rows<N, 4, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else if (R == 2) sweep_f64_rows<N, 2, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else sweep_f64_rows<N, 1, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
 }
 
 template <int N, int KIND>
