@@ -276,6 +276,7 @@ struct LaunchClass {
     int item_begin, item_count;
     int block, grid;
     int csize;           // FP64 CTA and global-memory groups: blocks per grid (grid: clusters)
+    int budget;          // FP64 CTA groups: shared memory a block may fill
     size_t smem;
     int smem_group;
     int glog;            // warp groups: log2 lanes per group
@@ -365,6 +366,7 @@ struct Plan {
     bool use_multi = true;  // launch strategy (the autotuner may switch it)
     int glog_delta = 0;     // warp groups: lanes per grid widened by 2^glog_delta (autotuned)
     bool lean = false;      // no spare global scratch (plan_host)
+    bool sparse = false;    // few of the grids will be solved (the FP64 re-solve)
     // streams and events that let a solve's launches overlap (none: one after
     // the other).  Two at most: each costs a plan 50 us, and more launches than
     // three at a time measured no faster.
@@ -414,6 +416,58 @@ int log2i(int v)
     int r = 0;
     while ((1 << (r + 1)) <= v) ++r;
     return r;
+}
+
+// Width of a class of FP64 grids on whole blocks in shared memory, by the time
+// its grids would take.  One block of up to 256 threads per SM finishes a grid
+// soonest; two of 128 or four of 64, each with its part of the shared memory,
+// hide each other's barriers and latency, and so take more grids per time.
+// Measured, as the time of all resident grids, 1 x 256 / 2 x 128 / 4 x 64 per
+// SM (8 steps, full grids): N=2 256 nodes 166 / 236 / 315 us, N=4 270 / 387 /
+// 497, N=8 522 / 758 / 1177; N=3 512 nodes 329 / 514 / 685; N=2 1024 nodes 439 /
+// 761 / 1041, N=5 836 / 1539 / 2860; 4096 nodes N=2 1.56 / 2.66 ms, N=3 1.66 /
+// 3.7, N=6 4.6 / 12.6.  The last three show where it ends: a part of the shared
+// memory in which a grid's differences or factors no longer fit loses or gains
+// nothing (N >= 3; two axes have one pair and few factors).  Grids of 128 nodes
+// run two or more blocks per SM as they are.  130 instances of N=2 level 8
+// (2210 grids): one block of 256 per SM 2.46 ms, these widths 1.08.
+template <class It>
+void f64_widths(LaunchClass& c, It first, It last, int lmax, int sms, bool lean)
+{
+    const int widest = c.block;
+    double work = 0.0;  // grids, in largest ones
+    for (It q = first; q != last; ++q) work += (double)q->L / lmax;
+    const bool equal = work == (double)c.item_count;
+    double best = 0.0;
+    for (int t = 1; t <= 4; t *= 2) {
+        const int block = std::min(widest, kCtaMaxThreads / t);
+        const int budget = t == 1 ? kF64SmemMax : kF64SmemMax / t - 1024;
+        int smem = 0;
+        int64_t slice = 0;
+        bool keeps = true;
+        for (It q = first; q != last; ++q) {
+            if (q != first && memcmp(q->it.lv, (q - 1)->it.lv, sizeof(q->it.lv)) == 0) continue;
+            const F64Layout y = f64_layout(c.N, q->it.lv, kCtaGroup, 1, block, budget, lean);
+            smem = std::max(smem, y.smem);
+            slice = std::max(slice, y.slice);
+            if (t > 1 && c.N > 2) {
+                const F64Layout w = f64_layout(c.N, q->it.lv, kCtaGroup, 1, widest, kF64SmemMax, lean);
+                keeps = keeps && (y.diff || !w.diff) && ((y.fast & 1) || !(w.fast & 1));
+            }
+        }
+        const int occ = occ_for(c.N)(false, kCtaGroup, block, (size_t)smem);
+        if (t > 1 && (occ < t || !keeps)) break;
+        // (scarce scratch: narrower blocks only while their slices take half of it)
+        if (t > 1 && lean && slice * std::min(c.item_count, occ * sms) > AMFRW_NOALLOC_SCRATCH_BYTES / 2) break;
+        const double rounds = work / ((double)std::max(1, occ) * sms);
+        const double cost = (rounds <= 1.0 ? 1.0 : (equal ? std::ceil(rounds) : std::max(2.0, rounds))) *
+                            (occ < 2 ? 1.0 : (occ < 4 ? (lmax <= 128 ? 1.05 : (lmax <= 256 ? 1.45 : 1.75))
+                                                      : (lmax <= 256 ? 2.1 : 2.5)));
+        if (t > 1 && cost >= best) continue;
+        best = cost;
+        c.block = block;
+        c.budget = budget;
+    }
 }
 
 // Host-side plan: validated instances, grid list grouped into launch classes
@@ -471,7 +525,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                 // the register sweeps take, keep their state in global memory
                 int bytes = lay.total;
                 if (!warp && !mixed) {  // FP64 on whole blocks: lines of any length
-                    bytes = f64_layout(N, g.lv, kCtaGroup, 1, lean).smem;
+                    bytes = f64_layout(N, g.lv, kCtaGroup, 1, kCtaMaxThreads, kF64SmemMax, lean).smem;
                     if (force_mem || bytes > std::min(smem_cap, kF64SmemMax)) {
                         kind = kMemGroup;
                         bytes = 0;
@@ -598,8 +652,10 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
             const bool mem = c.kind == kMemGroup;
             int b = 64;
             while (b < kCtaMaxThreads && b < lmax) b *= 2;
-            c.block = b;
             c.csize = 1;
+            c.block = b;
+            c.budget = kF64SmemMax;
+            if (!mem && !P.sparse) f64_widths(c, all.begin() + k, all.begin() + e, lmax, sms, lean);
             int rows = 1 << 30;  // of the axis a cluster splits, and lines along it: a share for every block
             for (size_t q = k; q < e; ++q) {
                 const int lx = all[q].it.lv[f64_split(c.N, all[q].it.lv)];
@@ -610,7 +666,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                 c.csize *= 2;
             int bytes = 0;
             for (size_t q = k; q < e; ++q) {
-                const F64Layout y = f64_layout(c.N, all[q].it.lv, c.kind, c.csize, lean);
+                const F64Layout y = f64_layout(c.N, all[q].it.lv, c.kind, c.csize, c.block, c.budget, lean);
                 bytes = std::max(bytes, y.smem);
                 lumax = std::max(lumax, y.slice);
             }
@@ -1037,6 +1093,7 @@ SolveArgs class_args(const Plan& P, const LaunchClass& L, int c, int steps, int 
     a.lu_stride = L.lu_stride;
     a.inst_mask = P.inst_mask;
     a.csize = std::max(1, L.csize);
+    a.budget = L.budget;
     if (P.lean) a.flags |= kLeanScratch;
     return a;
 }
@@ -1153,12 +1210,13 @@ int class_to_global(Plan& P, int c)
     for (int q = L.item_begin; q < L.item_begin + L.item_count; ++q) {
         const int8_t* lv = P.items[(size_t)q].lv;
         lumax = std::max<int64_t>(lumax, L.mixed ? make_layout(L.N, lv, true, kMemGroup, log2i(kMemBlock)).total
-                                                 : f64_layout(L.N, lv, kMemGroup, 1, P.lean).slice);
+                                                 : f64_layout(L.N, lv, kMemGroup, 1, kMemBlock, kF64SmemMax, P.lean).slice);
     }
     const int per_sm = occ_for(L.N)(L.mixed, kMemGroup, kMemBlock, 0);
     if (per_sm < 1) return fail(AMFRW_ETOOBIG, "no resident block possible for a global-memory class");
     L.kind = kMemGroup;
     L.csize = 1;
+    L.budget = kF64SmemMax;
     L.block = kMemBlock;
     L.smem = 0;
     L.lu_stride = (lumax + 255) & ~(int64_t)255;
@@ -1406,6 +1464,7 @@ int build_promotion(amfrw_batch* b, const amfrw_params* ps, int n, void* stream)
     b->promo.reset(new (std::nothrow) Plan());
     if (!b->promo) return fail(AMFRW_ENOMEM, "host allocation failed");
     Plan& Q = *b->promo;
+    Q.sparse = true;
     // (no bundles: few instances are re-solved, and a bundle costs what its
     // 32 lanes cost however few are marked)
     int st = build_plan(q.data(), n, stream, false, false, false, Q);

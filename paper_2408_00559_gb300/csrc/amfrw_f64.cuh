@@ -222,10 +222,10 @@ __device__ void solve_item_f64(const SolveArgs& a, const Item& it, unsigned char
     constexpr bool MEM = KIND == kMemGroup;
     const int nt = (int)blockDim.x, tid = (int)threadIdx.x;
     const bool lean = (a.flags & kLeanScratch) != 0;
-    const F64Layout y = f64_layout(N, it.lv, KIND, csize, lean);
+    const F64Layout y = f64_layout(N, it.lv, KIND, csize, nt, a.budget, lean);
     const InstDev& P = a.insts[it.inst];
     Shape<N> s;
-    make_shape<N>(s, it.lv, f64_tlog(csize), kRowsLogMem, true, true, P.bc != 0);
+    make_shape<N>(s, it.lv, f64_tlog(csize, nt), kRowsLogMem, true, true, P.bc != 0);
     unsigned char* base = MEM ? slice : smem;  // the vectors and the small tables
     double* cst = reinterpret_cast<double*>(base + y.cst);
     double* tabd = reinterpret_cast<double*>(base + y.tabd);

@@ -320,6 +320,7 @@ struct SolveArgs {
     // re-solve of ill-conditioned mixed-precision instances skips the others
     const int32_t* inst_mask;
     int32_t csize;        // FP64 CTA and global-memory groups: blocks per grid (a cluster)
+    int32_t budget;       // FP64 whole-block groups: f64_layout's
 };
 
 constexpr int kLoadState = 1;
@@ -338,11 +339,12 @@ constexpr int kMaxCluster = 8;
 // log2 of the lanes among which the lines of a solve are spread: all warps of
 // a block; half of a cluster's, whose lines are short enough by then (65x65
 // grid on eight blocks: 1.25 ms with a quarter, 1.04 with half).
-AMFRW_HD int f64_tlog(int csize)
+AMFRW_HD int f64_tlog(int csize, int block)
 {
-    int c = 0;
+    int c = 0, b = 0;
     while ((2 << c) <= csize) ++c;
-    return 8 + (c > 0 ? c - 1 : 0);
+    while ((2 << b) <= block) ++b;
+    return b + (c > 0 ? c - 1 : 0);
 }
 
 struct F64Layout {
@@ -370,7 +372,8 @@ AMFRW_HD bool f64_own_classes(int N, const int8_t* lv, int axis, int csize)
     return N == 2 && axis == 0 && csize > 1 && f64_split(N, lv) == 1;
 }
 
-AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, bool lean)
+// budget: shared memory a block of a CTA group may fill.
+AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, int block, int budget, bool lean)
 {
     F64Layout y{};
     int llog = 0, sumM = 0, npay = 0, ncx = 0;
@@ -390,7 +393,7 @@ AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, bool
         const int rows = (i < N - 1 ? MV : 1) << lv[i];
         rmax = rows > rmax ? rows : rmax;
         // (make_shape's line-solve region: folded axes keep their place)
-        const int64_t n = (int64_t)rows * lu_row_values(lanes_log(lv[i], llog, f64_tlog(csize), kRowsLogMem));
+        const int64_t n = (int64_t)rows * lu_row_values(lanes_log(lv[i], llog, f64_tlog(csize, block), kRowsLogMem));
         nlu += n;
         nlu_own += f64_own_classes(N, lv, i, csize) ? n / csize : n;
         if (i >= 1 && i < N - 1 && lv[i] > 0) ndr += 1 << (sh + lv[i] - lv[0]);
@@ -418,11 +421,11 @@ AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, bool
     y.K1 = small(8 * y.Lp);
     y.Kw = small(8 * y.Lp);
     const int64_t dbytes = (int64_t)8 * (N - 1) * y.Lp;
-    y.diff = mem ? (lean ? 0 : 1) : (csize == 1 && o + dbytes <= kF64SmemMax ? 1 : 0);
+    y.diff = mem ? (lean ? 0 : 1) : (csize == 1 && o + dbytes <= budget ? 1 : 0);
     y.D = y.diff ? small((int)dbytes) : 0;
     // in shared memory while it lasts, else in the slice
     auto rest = [&](int64_t fast_bytes, int64_t bytes, int bit) {
-        if (!mem && o + fast_bytes + 16 <= kF64SmemMax) {
+        if (!mem && o + fast_bytes + 16 <= budget) {
             y.fast |= bit;
             return small((int)fast_bytes);
         }
