@@ -276,7 +276,7 @@ struct LaunchClass {
     int item_begin, item_count;
     int block, grid;
     int csize;           // FP64 CTA and global-memory groups: blocks per grid (grid: clusters)
-    int budget;          // FP64 CTA groups: shared memory a block may fill
+    int budget;          // FP64 CTA groups: shared memory a block may fill; global-memory groups: 0 without differences
     size_t smem;
     int smem_group;
     int glog;            // warp groups: log2 lanes per group
@@ -468,6 +468,22 @@ void f64_widths(LaunchClass& c, It first, It last, int lmax, int sms, bool lean)
         c.block = block;
         c.budget = budget;
     }
+}
+
+// Whether grids with their state in global memory store central differences.
+// They save FP64 instructions but add a pass and N - 1 vectors to stream, so
+// they pay where the vectors stay in L2 or two blocks share an SM, and not
+// where memory is what the grids wait for (direct stencil / differences):
+// N=4, 2^16 nodes, 20 grids (74 MB) 6.00 / 5.60 ms, 60 grids (222 MB) 12.4 /
+// 13.3, 304 grids (two blocks per SM) 43.4 / 40.2; N=4, 2^20 nodes, one grid
+// (58 MB) 23.0 / 21.3 ms, 160 grids 337 / 464.  Two axes have one pair: the
+// direct stencil is never slower (2^20 nodes 13.7 / 14.2 ms).
+bool f64_mem_differences(const LaunchClass& c, int lmax, int64_t slice, int sms)
+{
+    if (c.N == 2) return false;
+    const int per_sm = std::max(1, occ_for(c.N)(false, kMemGroup, c.block, 0));
+    const int64_t blocks = std::min<int64_t>((int64_t)c.item_count * c.csize, (int64_t)per_sm * sms);
+    return slice * (blocks / c.csize) <= (int64_t)200 << 20 || (blocks > sms && lmax <= 1 << 16);
 }
 
 // Host-side plan: validated instances, grid list grouped into launch classes
@@ -665,10 +681,20 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                    lmax / (c.csize * 2) >= (mem ? 1024 : 128))
                 c.csize *= 2;
             int bytes = 0;
-            for (size_t q = k; q < e; ++q) {
-                const F64Layout y = f64_layout(c.N, all[q].it.lv, c.kind, c.csize, c.block, c.budget, lean);
-                bytes = std::max(bytes, y.smem);
-                lumax = std::max(lumax, y.slice);
+            auto sizes = [&]() {
+                bytes = 0;
+                lumax = 0;
+                for (size_t q = k; q < e; ++q) {
+                    if (q > k && memcmp(all[q].it.lv, all[q - 1].it.lv, sizeof(all[q].it.lv)) == 0) continue;
+                    const F64Layout y = f64_layout(c.N, all[q].it.lv, c.kind, c.csize, c.block, c.budget, lean);
+                    bytes = std::max(bytes, y.smem);
+                    lumax = std::max(lumax, y.slice);
+                }
+            };
+            sizes();
+            if (mem && !f64_mem_differences(c, lmax, lumax, sms)) {
+                c.budget = 0;
+                sizes();
             }
             c.smem = mem ? 0 : (size_t)bytes;
         } else if (c.kind == kCtaGroup) {

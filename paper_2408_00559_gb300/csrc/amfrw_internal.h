@@ -372,7 +372,8 @@ AMFRW_HD bool f64_own_classes(int N, const int8_t* lv, int axis, int csize)
     return N == 2 && axis == 0 && csize > 1 && f64_split(N, lv) == 1;
 }
 
-// budget: shared memory a block of a CTA group may fill.
+// budget: shared memory a block of a CTA group may fill; 0 for global-memory
+// groups without stored differences.
 AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, int block, int budget, bool lean)
 {
     F64Layout y{};
@@ -421,7 +422,7 @@ AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, int 
     y.K1 = small(8 * y.Lp);
     y.Kw = small(8 * y.Lp);
     const int64_t dbytes = (int64_t)8 * (N - 1) * y.Lp;
-    y.diff = mem ? (lean ? 0 : 1) : (csize == 1 && o + dbytes <= budget ? 1 : 0);
+    y.diff = mem ? (lean || budget == 0 ? 0 : 1) : (csize == 1 && o + dbytes <= budget ? 1 : 0);
     y.D = y.diff ? small((int)dbytes) : 0;
     // in shared memory while it lasts, else in the slice
     auto rest = [&](int64_t fast_bytes, int64_t bytes, int bit) {
