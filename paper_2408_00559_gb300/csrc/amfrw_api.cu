@@ -553,6 +553,20 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                 }
                 gi.push_back(GridInfo{g, lay.L, kind, warp, bytes, 0});
             }
+            // A call whose launches run one by one (lean) solves lines of more
+            // than 256 rows, which wait for memory wherever they lie, beside the
+            // grids that have to be in global memory, if there are any (N=2
+            // level 12, six steps: 7.8 -> 4.6 ms; without such grids the
+            // launch more costs up to 1.6 times).
+            bool any_mem = false;
+            for (const GridInfo& x : gi) any_mem |= x.kind == kMemGroup;
+            for (GridInfo& x : gi) {
+                const int8_t most = *std::max_element(x.g.lv, x.g.lv + N);
+                if (lean && !mixed && any_mem && x.kind == kCtaGroup && most > 8) {
+                    x.kind = kMemGroup;
+                    x.smem_group = 0;
+                }
+            }
             it = shapes.emplace(id, std::move(gi)).first;
         }
         inst_shape[(size_t)i] = &it->second;
