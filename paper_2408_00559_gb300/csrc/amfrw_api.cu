@@ -437,26 +437,29 @@ void f64_widths(LaunchClass& c, It first, It last, int lmax, int sms, bool lean)
     const int widest = c.block;
     double work = 0.0;  // grids, in largest ones
     for (It q = first; q != last; ++q) work += (double)q->L / lmax;
+    if (work <= sms) return;  // one block per SM takes them in one round
     const bool equal = work == (double)c.item_count;
+    const int64_t stride = std::max<int64_t>(1, (last - first) / 32);  // (some of the grids, for speed)
     double best = 0.0;
     for (int t = 1; t <= 4; t *= 2) {
         const int block = std::min(widest, kCtaMaxThreads / t);
+        if (t > 1 && block == widest) continue;
         const int budget = t == 1 ? kF64SmemMax : kF64SmemMax / t - 1024;
         int smem = 0;
         int64_t slice = 0;
         bool keeps = true;
-        for (It q = first; q != last; ++q) {
-            if (q != first && memcmp(q->it.lv, (q - 1)->it.lv, sizeof(q->it.lv)) == 0) continue;
+        for (It q = first; q < last && keeps; q += std::min<int64_t>(stride, last - q)) {
             const F64Layout y = f64_layout(c.N, q->it.lv, kCtaGroup, 1, block, budget, lean);
             smem = std::max(smem, y.smem);
             slice = std::max(slice, y.slice);
-            if (t > 1 && c.N > 2) {
+            if (t > 1 && c.N > 2 && (!y.diff || !(y.fast & 1))) {
                 const F64Layout w = f64_layout(c.N, q->it.lv, kCtaGroup, 1, widest, kF64SmemMax, lean);
-                keeps = keeps && (y.diff || !w.diff) && ((y.fast & 1) || !(w.fast & 1));
+                keeps = (y.diff || !w.diff) && ((y.fast & 1) || !(w.fast & 1));
             }
         }
+        if (!keeps) break;
         const int occ = occ_for(c.N)(false, kCtaGroup, block, (size_t)smem);
-        if (t > 1 && (occ < t || !keeps)) break;
+        if (t > 1 && occ < t) break;
         // (scarce scratch: narrower blocks only while their slices take half of it)
         if (t > 1 && lean && slice * std::min(c.item_count, occ * sms) > AMFRW_NOALLOC_SCRATCH_BYTES / 2) break;
         const double rounds = work / ((double)std::max(1, occ) * sms);
@@ -535,23 +538,23 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
                 const bool warp = (1 << llog) <= kWarpMaxL && !force_mem;
                 // warp groups: two nodes per lane, so small grids share a warp
                 int kind = warp ? kWarpGroup : kCtaGroup;
-                Layout lay = make_layout(N, g.lv, mixed, kind,
-                                         warp ? warp_group_log(llog, mixed) : 5);
+                int bytes = 0;
                 // grids beyond shared memory, or (mixed) with lines longer than
                 // the register sweeps take, keep their state in global memory
-                int bytes = lay.total;
                 if (!warp && !mixed) {  // FP64 on whole blocks: lines of any length
                     bytes = f64_layout(N, g.lv, kCtaGroup, 1, kCtaMaxThreads, kF64SmemMax, lean).smem;
                     if (force_mem || bytes > std::min(smem_cap, kF64SmemMax)) {
                         kind = kMemGroup;
                         bytes = 0;
                     }
-                } else if (force_mem || lay.total > smem_cap || (!warp && maxlv > 5 + rows_log(kCtaGroup))) {
-                    kind = kMemGroup;
-                    lay = make_layout(N, g.lv, mixed, kind, log2i(kMemBlock));
-                    bytes = lay.total;
+                } else {
+                    bytes = make_layout(N, g.lv, mixed, kind, warp ? warp_group_log(llog, mixed) : 5).total;
+                    if (force_mem || bytes > smem_cap || (!warp && maxlv > 5 + rows_log(kCtaGroup))) {
+                        kind = kMemGroup;
+                        bytes = make_layout(N, g.lv, mixed, kind, log2i(kMemBlock)).total;
+                    }
                 }
-                gi.push_back(GridInfo{g, lay.L, kind, warp, bytes, 0});
+                gi.push_back(GridInfo{g, 1 << llog, kind, warp, bytes, 0});
             }
             // A call whose launches run one by one (lean) solves lines of more
             // than 256 rows, which wait for memory wherever they lie, beside the
