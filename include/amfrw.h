@@ -284,7 +284,9 @@ void amfrw_batch_destroy(amfrw_batch *b);
  * DEVICE, row-major BF16 with leading dimensions lda, ldb (multiples of 8,
  * >= K, 16-byte aligned); C: DEVICE FP32 row-major with leading dimension
  * ldc >= N.  Requires N a multiple of 16 (and of 256 when above 256), K a
- * multiple of 16.  Synchronises.  Errors: EINVAL, ENOMEM, ECUDA, ETIMEOUT
+ * multiple of 16.  Synchronises.  A thread's first call allocates a word of
+ * pinned host memory, freed when the thread ends; later calls allocate
+ * nothing.  Errors: EINVAL, ENOMEM, ECUDA, ETIMEOUT
  * (a bounded wait inside the kernel gave up; the result is not valid). */
 int amfrw_tc_gemm_bf16(const void *dA, int32_t lda, const void *dB, int32_t ldb, float *dC,
                        int32_t ldc, int32_t M, int32_t N, int32_t K, void *cuda_stream);

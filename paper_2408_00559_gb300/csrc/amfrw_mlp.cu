@@ -49,8 +49,24 @@ bool make_map(CUtensorMap* tm, const __nv_bfloat16* base, int rows, int K, int l
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// SMs of the current device and the launch limits of its kernels, set once per
-// device.
+// Identity of the current context, unique over the life of the process: what
+// belongs to a context (pinned memory, kernel attributes) is gone after a
+// device reset, although device numbers and addresses come back.  0: none.
+unsigned long long context_id()
+{
+    using Fn = CUresult (*)(CUcontext, unsigned long long*);
+    static const Fn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return ok ? (Fn)p : nullptr;
+    }();
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// SMs of the current device.
 int device_sms(int dev)
 {
     static std::atomic<int> sms[64];
@@ -87,19 +103,22 @@ int tile_stages(int BN, int nk, int tiles, int sms)
     return S;
 }
 
-// Raises the kernels' dynamic shared-memory limit, an attribute per device,
-// once on every device that launches them (to the most any launch asks for).
-int raise_limits(int dev)
+// Raises the kernels' dynamic shared-memory limit, an attribute per context,
+// once on every device that launches them (to the most any launch asks for),
+// when a launch needs more than every kernel may have.
+int raise_limits(int dev, int smem)
 {
+    if (smem <= 48 * 1024) return 0;
     static std::mutex mu;
-    static bool attr[64] = {};
+    static unsigned long long attr[64] = {};  // context whose limits are raised
+    const unsigned long long ctx = context_id();
     std::lock_guard<std::mutex> lock(mu);
-    if (!attr[dev]) {
+    if (ctx == 0 || attr[dev] != ctx) {
         const int most = 200 * 1024 + 1024;
         cudaError_t e = cudaFuncSetAttribute(gemm_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return (int)e;
-        attr[dev] = true;
+        attr[dev] = ctx;
     }
     return 0;
 }
@@ -118,7 +137,7 @@ int gemm(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M
     const int BN = epi.mode == 3 ? (N <= 256 ? N : 256) : tile_columns(M, N, sms);
     const dim3 grid((M + kBM - 1) / kBM, (N + BN - 1) / BN);
     const int S = tile_stages(BN, (K + kBK - 1) / kBK, grid.x * grid.y, sms);
-    if (const int rc = raise_limits(dev)) return rc;
+    if (const int rc = raise_limits(dev, smem_bytes(BN, S))) return rc;
     CUtensorMap tA, tB;
     if (!make_map(&tA, A, M, K, lda, kBM) || !make_map(&tB, B, N, K, ldb, BN)) return (int)cudaErrorInvalidValue;
     gemm_bf16_kernel<<<grid, kThreads, smem_bytes(BN, S), st>>>(tA, tB, M, N, K, BN, S, epi);
@@ -155,7 +174,7 @@ int gemm3(const Product (&p)[3], int lda, int ldb, int K, int* error, cudaStream
             return (int)cudaErrorInvalidValue;
     }
     j.S = tile_stages(wide, (K + kBK - 1) / kBK, j.first[3], sms);
-    if (const int rc = raise_limits(dev)) return rc;
+    if (const int rc = raise_limits(dev, smem_bytes(wide, j.S))) return rc;
     gemm_bf16_batch_kernel<<<j.first[3], kThreads, smem_bytes(wide, j.S), st>>>(j);
     return (int)cudaGetLastError();
 }
@@ -166,17 +185,32 @@ int gemm3(const Product (&p)[3], int lda, int ldb, int K, int* error, cudaStream
 using namespace amfrw;
 
 namespace {
-// A word of pinned host memory that every device can write.
-struct HostFlag {
-    int* p = nullptr;
-    bool get()
+// A thread's words of pinned host memory, one per context it has used: a word
+// of a context that a device reset ended is neither written nor freed.
+struct HostWords {
+    struct Word {
+        unsigned long long ctx;
+        int* p;
+    };
+    Word w[16] = {};
+    int n = 0;
+    int* get()
     {
-        if (!p && cudaHostAlloc(&p, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) p = nullptr;
-        return p != nullptr;
+        const unsigned long long ctx = tc::context_id();
+        if (ctx == 0) return nullptr;
+        for (const Word& x : w)
+            if (x.p && x.ctx == ctx) return x.p;
+        int* p = nullptr;
+        if (cudaHostAlloc(&p, sizeof(int), cudaHostAllocMapped) != cudaSuccess) return nullptr;
+        w[n++ % 16] = Word{ctx, p};
+        return p;
     }
-    ~HostFlag()
+    ~HostWords()
     {
-        if (p) cudaFreeHost(p);
+        if (n == 0) return;
+        const unsigned long long ctx = tc::context_id();
+        for (const Word& x : w)
+            if (x.p && x.ctx == ctx) cudaFreeHost(x.p);
     }
 };
 }  // namespace
@@ -192,21 +226,23 @@ extern "C" int amfrw_tc_gemm_bf16(const void* dA, int32_t lda, const void* dB, i
     // A call waits for its result, so it cannot be recorded into a graph.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return AMFRW_ECUDA;
-    // The kernel's error word: one per calling thread in pinned host memory
-    // (a thread has one call in flight), written only when a wait gives up, so
-    // that a call neither allocates nor copies.
-    thread_local HostFlag flag;
-    if (!flag.get()) return AMFRW_ENOMEM;
-    *flag.p = 0;
+    // The kernel's error word: one per calling thread and context in pinned host
+    // memory (a thread has one call in flight), written only when a wait gives
+    // up, so that a call neither allocates nor copies (a thread's first allocates
+    // the word).
+    thread_local HostWords words;
+    int* word = words.get();
+    if (!word) return AMFRW_ENOMEM;
+    *word = 0;
     tc::Epi e{};
     e.mode = 0;
     e.C = dC;
     e.ldc = ldc;
-    e.error = flag.p;
+    e.error = word;
     int rc = tc::gemm((const __nv_bfloat16*)dA, lda, (const __nv_bfloat16*)dB, ldb, M, N, K, e, st);
     if (rc == 0) rc = (int)cudaStreamSynchronize(st);
     if (rc != 0) return AMFRW_ECUDA;
-    return *flag.p ? AMFRW_ETIMEOUT : AMFRW_OK;
+    return *word ? AMFRW_ETIMEOUT : AMFRW_OK;
 }
 
 // ===========================================================================
