@@ -1062,8 +1062,10 @@ int build_plan(const amfrw_params* ps, int n, void* stream, bool keep_state, boo
     CUDA_TRY(cudaMemsetAsync(P.d_u, 0, sizeof(double) * P.coefs.size(), P.stream));
     if (overlap && launch_records(P).size() > 1) {
         P.sides = std::min((int)launch_records(P).size() - 1, Plan::kSides);
+        int priority = 0;  // the caller's
+        CUDA_TRY(cudaStreamGetPriority(P.stream, &priority));
         for (int q = 0; q < P.sides; ++q) {
-            CUDA_TRY(cudaStreamCreateWithFlags(&P.side[q], cudaStreamNonBlocking));
+            CUDA_TRY(cudaStreamCreateWithPriority(&P.side[q], cudaStreamNonBlocking, priority));
             CUDA_TRY(cudaEventCreateWithFlags(&P.join[q], cudaEventDisableTiming));
         }
         CUDA_TRY(cudaEventCreateWithFlags(&P.fork, cudaEventDisableTiming));
