@@ -120,8 +120,9 @@ constexpr int kPairLr = 8, kPairLq = 16;                             // neighbou
 // Mixed precision (T float): stencil_act2's terms in its order, every product
 // fused as there (explicitly: across branches the compiler does not), with
 // zeros for Outer neighbours, acc starting as the single-row axes' term.  FP64:
-// neighbour sums, a term for each neighbour that is not Outer, acc starting
-// with the centre term.
+// second differences on axes of four rows or more and outside the block,
+// neighbour sums on the block's axes of two rows (acc starts with their and the
+// single-row axes' centre term), a term for each neighbour that is not Outer.
 template <typename T, bool PAIR, int PAT>
 __device__ __forceinline__ void block_F(const unsigned char* sm, int pc, int n, int xs, int at, int zero, int tb, int halos,
                                         const typename BundleSrc<T, PAIR>::V (&x)[Pat<PAT>::NB], T (&acc)[Pat<PAT>::NB])
@@ -1111,8 +1112,8 @@ __device__ void solve_bundle(const BundleArgs& a, const Bundle bd, int tlog, uns
 }
 
 // Persistent launch over bundle classes in descending group size: a block's
-// eight warps form one group for grids of 64 nodes, two of four warps for 32,
-// four of two for the rest.  A group takes bundles from its class's counter
+// eight warps form one group for grids of 64 nodes, two of four warps for the
+// rest.  A group takes bundles from its class's counter
 // until none is left, then goes on to the next class, splitting where that
 // class's groups are smaller.
 template <int N, bool MIXED>

@@ -176,11 +176,11 @@ AMFRW_HD bool dense_axis(int kind, bool mixed, int M)
 // 2 or more.
 AMFRW_HD int pad_rows_min(bool lean) { return lean ? 4 : 2; }
 
-// kind: the work-group kind.  Warp and global-memory groups keep the
-// line-solve factors inside the layout; CTA groups in the group's slice of a
-// global scratch array.  Global-memory groups also get FP64 scratch for the
-// factorisation (three values per matrix row of the largest axis).  tlog:
-// log2 of the group's thread count.
+// kind: the work-group kind (FP64: warp groups only; whole blocks have
+// f64_layout).  Warp and global-memory groups keep the line-solve factors inside
+// the layout; CTA groups in the group's slice of a global scratch array.
+// Global-memory groups also get FP64 scratch for the factorisation (three values
+// per matrix row of the largest axis).  tlog: log2 of the group's thread count.
 AMFRW_HD Layout make_layout(int N, const int8_t* lv, bool mixed, int kind, int tlog)
 {
     Layout y{};
@@ -220,7 +220,6 @@ AMFRW_HD Layout make_layout(int N, const int8_t* lv, bool mixed, int kind, int t
     }
     const bool lu_in = kind != kCtaGroup;
     y.nlu = nlu;
-    const int sk = mixed ? 4 : 8;  // bytes of a factor value
     int o = 0;
     if (mixed) {
         // The FP64 constants and tables serve the per-grid setup only (tables,
@@ -258,7 +257,7 @@ AMFRW_HD Layout make_layout(int N, const int8_t* lv, bool mixed, int kind, int t
         y.tabd = o; o = align16(o + 8 * y.ntab);
         y.tabf = o;
         y.pay = o;  o = align16(o + 8 * y.npay);
-        y.lu = o;   o = align16(o + (lu_in ? 8 * y.nlu : 0));
+        y.lu = o;   o = align16(o + 8 * y.nlu);
         y.Z = o;    o = align16(o + 8 * y.Lp);
         y.ZZ = o;
         y.H = o;    o = align16(o + 8 * y.Lr);
@@ -267,10 +266,9 @@ AMFRW_HD Layout make_layout(int N, const int8_t* lv, bool mixed, int kind, int t
         y.K1 = o;   o = align16(o + 8 * y.Lp);
         y.K0 = o;   o = align16(o + 8 * y.Lp);
         y.Kw = o;   o = align16(o + 8 * y.Lp);
-        // FP64 warp groups: central differences per axis and per-node coefficients
-        const bool diff = kind == kWarpGroup;
-        y.ncoef = diff ? node_coefs(N) : 0;
-        y.D = o;    o = align16(o + (diff ? 8 * N * y.Lp : 0));
+        // central differences per axis and per-node coefficients
+        y.ncoef = node_coefs(N);
+        y.D = o;    o = align16(o + 8 * N * y.Lp);
         y.C = o;    o = align16(o + 8 * y.ncoef * y.Lp);
     }
     int rmax = 0;
@@ -280,14 +278,12 @@ AMFRW_HD Layout make_layout(int N, const int8_t* lv, bool mixed, int kind, int t
     }
     y.scr = o;  o = align16(o + (kind == kMemGroup ? 3 * 8 * rmax : 0));
     y.total = o;
-    // the global slice of a CTA group: factors, then (mixed) Z and dt F(Y_n)
+    // the global slice of a CTA group: factors, then Z and dt F(Y_n)
     y.gbytes = y.gZ = y.gFY = 0;
-    if (kind == kCtaGroup) {
-        int g = (nlu * sk + 255) & ~255;
-        if (lean) {
-            y.gZ = g;   g += (8 * y.Lp + 255) & ~255;
-            y.gFY = g;  g += (4 * y.Lp + 255) & ~255;
-        }
+    if (lean) {
+        int g = (4 * nlu + 255) & ~255;
+        y.gZ = g;   g += (8 * y.Lp + 255) & ~255;
+        y.gFY = g;  g += (4 * y.Lp + 255) & ~255;
         y.gbytes = g;
     }
     return y;
@@ -379,11 +375,9 @@ AMFRW_HD F64Layout f64_layout(int N, const int8_t* lv, int kind, int csize, int 
     F64Layout y{};
     int llog = 0, sumM = 0, npay = 0, ncx = 0;
     for (int i = 0; i < N; ++i) llog += lv[i];
-    bool rate_rows = false;
     for (int i = 0; i < N - 1; ++i) {
         sumM += 1 << lv[i];
         npay += (1 << lv[i]) + 1;
-        rate_rows |= lv[i] > 0;
         for (int k = i + 1; k < N; ++k) ncx += k < N - 1 ? 1 << lv[k] : 1;
     }
     const int MV = 1 << lv[N - 1], L = 1 << llog, Lr = L >> lv[N - 1];

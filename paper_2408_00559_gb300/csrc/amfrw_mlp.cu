@@ -743,15 +743,16 @@ struct amfrw_surrogate {
 
 namespace {
 
-// Buffers of one pass set: forward rows (activations) and training rows
-// (transposes, pre-activations, gradients).
+// Buffers of one pass set: forward rows (activations) and training rows (the
+// third layer's, which predictions do not store; transposes, pre-activations,
+// gradients).
 int sg_work_alloc(SgWork& w, size_t fwd_rows, size_t train_rows)
 {
     const size_t B2 = sizeof(bf16), F4 = sizeof(float);
     SG_CUDA(cudaMalloc(&w.X, B2 * fwd_rows * kInPad));
     SG_CUDA(cudaMalloc(&w.Xt, B2 * train_rows * kInPad));
-    for (bf16** q : {&w.H1, &w.H2, &w.H3}) SG_CUDA(cudaMalloc(q, B2 * fwd_rows * kW));
-    for (bf16** q : {&w.H1t, &w.H2t, &w.dZ1, &w.dZ2, &w.dZ3, &w.dZ1t, &w.dZ2t, &w.dZ3t})
+    for (bf16** q : {&w.H1, &w.H2}) SG_CUDA(cudaMalloc(q, B2 * fwd_rows * kW));
+    for (bf16** q : {&w.H3, &w.H1t, &w.H2t, &w.dZ1, &w.dZ2, &w.dZ3, &w.dZ1t, &w.dZ2t, &w.dZ3t})
         SG_CUDA(cudaMalloc(q, B2 * train_rows * kW));
     for (float** q : {&w.Z1, &w.Z2, &w.Z3}) SG_CUDA(cudaMalloc(q, F4 * train_rows * kW));
     SG_CUDA(cudaMalloc(&w.t, F4 * train_rows));
@@ -818,7 +819,7 @@ int sg_forward(amfrw_surrogate* s, int m, int B, bool train, float* y, const SgW
     int rc = tc::gemm(w.X, kInPad, s->W1b[m], kInPad, B, kW, kInPad, e, st);
     e.bias = s->P[m] + ob2; e.Z = train ? w.Z2 : nullptr; e.H = w.H2; e.Ht = train ? w.H2t : nullptr;
     if (!rc) rc = tc::gemm(w.H1, kW, s->W2b[m], kW, B, kW, kW, e, st);
-    e.bias = s->P[m] + ob3; e.Z = train ? w.Z3 : nullptr; e.H = w.H3; e.Ht = nullptr;
+    e.bias = s->P[m] + ob3; e.Z = train ? w.Z3 : nullptr; e.H = train ? w.H3 : nullptr; e.Ht = nullptr;
     // a prediction needs the third layer's activations only in its output,
     // which the product's epilogue forms (out_kernel's sum in its order)
     e.mode = train ? 1 : 3;

@@ -5,7 +5,7 @@
 //                                             FP32 accumulation in TMEM)
 //
 // One CTA of 256 threads computes a 128 x BN tile (BN <= 256, a multiple of
-// 16).  K advances in chunks of 64 through a ring of up to four shared-memory
+// 16).  K advances in chunks of 64 through a ring of up to eight shared-memory
 // stages filled by TMA: one box of 64 elements of K (128 bytes, the 128-byte
 // swizzle's span) by all rows per operand, in the swizzled K-major layout
 // (8 rows x 128 bytes per swizzle atom, atoms 1024 bytes apart along M/N).
