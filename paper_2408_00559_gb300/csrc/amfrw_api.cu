@@ -299,21 +299,12 @@ constexpr int kBundleMinMixed = 11;
 constexpr int kBundleMinF64 = 17;
 // A bundle takes 1.6 ms (mixed) or 2.4 ms (FP64) for 40 steps however few run
 // at once, which the warp groups beat on small batches: bundles where the
-// (N, precision) has at least this many Inner nodes per SM; lmax: its largest
-// warp-solved grid.  Measured crossovers, in nodes per SM: mixed 2 600 to 4 000
-// for every N (level 5 N=3 2 600, N=4 2 400, N=5 2 000; level 6 N=3 3 100, N=6
-// 3 900).  FP64: N=3 level 4 900, level 5 2 100, level 6 4 500; N=4 level 5
-// 1 200, level 6 1 700; N=5 level 5 900; from N=6 on below the fewest instances
-// a bundle takes.  N=2 in FP64 gains nothing at any size (bundles / warp groups
-// at 40 000 nodes per SM 1.06 to 1.14): its warp groups leave few lanes idle.
-constexpr int64_t kNeverBundled = (int64_t)1 << 60;
-int64_t bundle_nodes_per_sm(int N, bool mixed, int lmax)
-{
-    if (mixed) return 4000;
-    if (N == 2) return kNeverBundled;
-    if (N == 3) return lmax <= 32 ? 2100 : 4500;
-    return N == 4 && lmax > 32 ? 1700 : 1300;
-}
+// (N, precision) has at least this many Inner nodes per SM.  Measured
+// crossovers, in instances (nodes per SM): mixed N=3 level 5 550 (3 700), N=4
+// level 5 200 (3 400), N=6 level 6 20 (5 300), N=8 level 5 19 (4 000); FP64
+// N=3 level 5 310 (2 100), N=4 level 5 75 (1 250), N=6 level 5 10 (700).
+constexpr int64_t kBundleNodesMixed = 4000;
+constexpr int64_t kBundleNodesF64 = 1300;
 
 // Global-memory groups: at most this much scratch per launch class (it bounds
 // the number of resident blocks, each holding one grid's state).
@@ -656,14 +647,9 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
     P.n_grids = (int)P.coefs.size();
     P.state_len = state_off;
     const int sms = num_sms();
-    // Inner nodes of the warp-solved grids per (N, precision), all and the largest grid's
-    int64_t warp_nodes[kMaxDim + 1][2] = {};
-    int warp_lmax[kMaxDim + 1][2] = {};
+    int64_t warp_nodes[kMaxDim + 1][2] = {};  // Inner nodes of the warp-solved grids per (N, precision)
     for (const Tmp& t : all)
-        if (t.warp) {
-            warp_nodes[t.N][t.mixed ? 1 : 0] += t.L;
-            warp_lmax[t.N][t.mixed ? 1 : 0] = std::max(warp_lmax[t.N][t.mixed ? 1 : 0], t.L);
-        }
+        if (t.warp) warp_nodes[t.N][t.mixed ? 1 : 0] += t.L;
     for (size_t k = 0; k < all.size();) {
         size_t e = k;
         int gmax = 0, lmax = 0;
@@ -756,8 +742,7 @@ int plan_host(const amfrw_params* ps, int n, bool keep_state, bool bundles, bool
         P.lu_scratch_len += c.lu_stride * c.grid;
         c.bundle_begin = (int)P.bundles.size();
         c.rest_begin = c.item_begin;
-        if (c.warp && bundles &&
-            warp_nodes[c.N][c.mixed ? 1 : 0] / sms >= bundle_nodes_per_sm(c.N, c.mixed, warp_lmax[c.N][c.mixed ? 1 : 0])) {
+        if (c.warp && bundles && warp_nodes[c.N][c.mixed ? 1 : 0] >= sms * (c.mixed ? kBundleNodesMixed : kBundleNodesF64)) {
             // runs of equal levels (adjacent, in instance order): whole
             // bundles of the instances with Neumann faces, then what is left
             std::vector<Item> rest;

@@ -102,11 +102,7 @@ __global__ void __launch_bounds__(KIND == kWarpGroup ? 128 : kCtaMaxThreads, KIN
 template <int N>
 const void* kernel_for(bool mixed, int kind)
 {
-    if (kind == kBundle) {
-        if constexpr (N > 2)  // (N = 2 has none in FP64)
-            if (!mixed) return (const void*)bundle_kernel<N, false>;
-        return (const void*)bundle_kernel<N, true>;
-    }
+    if (kind == kBundle) return mixed ? (const void*)bundle_kernel<N, true> : (const void*)bundle_kernel<N, false>;
     if (kind == kWarpGroup)
         return mixed ? (const void*)solve_kernel<N, true, kWarpGroup> : (const void*)solve_kernel<N, false, kWarpGroup>;
     if (kind == kCtaGroup)
@@ -146,8 +142,7 @@ template <int N>
 int launch_bundle_impl(const BundleArgs& a, bool mixed, int grid, size_t smem, void* stream)
 {
     if (mixed) bundle_kernel<N, true><<<grid, kBundleThreads, smem, (cudaStream_t)stream>>>(a);
-    else if constexpr (N > 2) bundle_kernel<N, false><<<grid, kBundleThreads, smem, (cudaStream_t)stream>>>(a);
-    else return (int)cudaErrorInvalidValue;  // (never planned)
+    else bundle_kernel<N, false><<<grid, kBundleThreads, smem, (cudaStream_t)stream>>>(a);
     return (int)cudaGetLastError();
 }
 

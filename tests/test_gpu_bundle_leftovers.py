@@ -4,10 +4,9 @@ bundles do run (a batch with both has one launch more than one without).
 
 What is left to the warp groups: three instances beyond the last full bundle,
 and instances with Dirichlet faces, alternating with the others or most of the
-book.  Counts follow the rule (4000 Inner nodes per SM in mixed precision; in
-FP64 1300, more for three and four axes with grids of 64 nodes).  Prices: a
-component value may move by a few ulps of FP64 (64 of them allowed), the price
-by kappa = sum |c_l u_l| / |price| times that.
+book.  Counts follow the rule (4000 Inner nodes per SM in mixed precision, 1300
+in FP64).  Prices: a component value may move by a few ulps of FP64 (64 of them
+allowed), the price by kappa = sum |c_l u_l| / |price| times that.
 """
 import numpy as np
 import pytest
@@ -18,13 +17,7 @@ from paper_2408_00559_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-
-def nodes_per_sm(N, precision, largest):
-    if precision == "mixed":
-        return 4000
-    if N == 3:
-        return 2100 if largest <= 32 else 4500
-    return 1700 if N == 4 and largest > 32 else 1300
+NODES_PER_SM = {"mixed": 4000, "fp64": 1300}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -49,9 +42,8 @@ def enough(N, level, precision):
     prob = B.Problem(W.small_instance(N, level, steps=1, precision=precision))
     sizes = 2 ** prob.grid_info()[0].sum(axis=1)
     prob.close()
-    sizes = sizes[sizes <= 64]
-    need = nodes_per_sm(N, precision, int(sizes.max())) * torch.cuda.get_device_properties(0).multi_processor_count
-    return -(-need // int(sizes.sum())) // 32 * 32 + 32
+    need = NODES_PER_SM[precision] * torch.cuda.get_device_properties(0).multi_processor_count
+    return -(-need // int(sizes[sizes <= 64].sum())) // 32 * 32 + 32
 
 
 def run(insts):
@@ -98,13 +90,6 @@ def test_bundles_with_leftovers(N, level, precision):
     prices, n = run(insts)
     assert n == 3, n  # bundles, the three left over, the combination
     check(insts, prices, (0, 31, count // 2, count - 4, count - 1))
-
-
-def test_two_axes_in_fp64_are_not_bundled():
-    insts = instances(2, 5, 1507, "fp64", neumann)  # (bundles would leave three)
-    prices, n = run(insts)
-    assert n == 2, n
-    check(insts, prices, (0, 1506))
 
 
 @pytest.mark.parametrize("N,level,precision", [(3, 5, "mixed"), (4, 5, "fp64")])
