@@ -299,10 +299,16 @@ constexpr int kBundleMinMixed = 11;
 constexpr int kBundleMinF64 = 17;
 // A bundle takes 1.6 ms (mixed) or 2.4 ms (FP64) for 40 steps however few run
 // at once, which the warp groups beat on small batches: bundles where the
-// (N, precision) has at least this many Inner nodes per SM.  Measured
-// crossovers, in instances (nodes per SM): mixed N=3 level 5 550 (3 700), N=4
-// level 5 200 (3 400), N=6 level 6 20 (5 300), N=8 level 5 19 (4 000); FP64
-// N=3 level 5 310 (2 100), N=4 level 5 75 (1 250), N=6 level 5 10 (700).
+// (N, precision) has at least this many Inner nodes per SM, all its warp-solved
+// grids counted (few bundles of a long book hide behind its warp groups: 400
+// Dirichlet and 17 other d=4 level-5 instances 11.6 ms with bundles, 11.8
+// without).  Measured crossovers in nodes per SM: mixed 2 000 to 4 000 for every
+// N; FP64 N=4 level 5 1 200, level 6 1 700, N=5 level 5 900, from N=6 on below
+// the fewest instances a bundle takes.  For N=3 they lie higher (level 5 2 100,
+// level 6 4 500) and for N=2 the warp groups stay faster (22 000 instances of
+// level 5, ten steps: 9.6 against 10.1 ms), but bundles are closer to an extended-precision solve (rms
+// relative error of a price, warp groups / bundles: N=3 level 6 7.9e-15 /
+// 9.1e-16, N=2 level 6 2.5e-14 / 3.6e-16), so the line is the same for every N.
 constexpr int64_t kBundleNodesMixed = 4000;
 constexpr int64_t kBundleNodesF64 = 1300;
 

@@ -16,17 +16,22 @@
 //    of cyclic reduction costs two instructions a row, elimination three), its
 //    rows streamed from memory instead of held in registers, so a line may
 //    have any length.
-// A launch with fewer grids than SMs gives each a cluster.  A block owns a slab
+// A class with at most half as many grids as SMs gives each a cluster, if every
+// one of its grids has enough lines and rows along its longest axis for the
+// blocks (a class that holds a grid of one line, as the largest grids of a
+// standard combination do, runs a block per grid).  A block owns a slab
 // of rows of the longest axis: it evaluates the stencil there and solves the
 // other axes' lines, which lie inside the slab; rows at the slab's edges are
 // stored into the neighbour's copy too.  Lines along the split axis are shared
 // out; their values come from and go back to the owners through distributed
 // shared memory.
-// Measured: 65x65 full grid, 20 steps, 4.31 -> 1.10 ms (eight blocks); 120 grids
-// of 128 nodes, 10 steps, 0.46 -> 0.28 ms; a d=4 level-12 combination, 8 steps:
-// its 450 grids of 4096 nodes 13.35 -> 13.3 ms (the rest of the time is
-// shared-memory and FP64 latency with eight warps per SM), its five grids with
-// the state in global memory 9.4 -> 7.8 ms.
+// A class with more grids than SMs runs one, two or four blocks per SM, each
+// with its part of the shared memory (f64_widths in amfrw_api.cu).
+// Measured, before this kernel -> now: 65x65 full grid, 20 steps, 4.31 -> 0.94
+// ms (eight blocks); 120 grids of 128 nodes, 10 steps, 0.46 -> 0.24 ms; a d=4
+// level-12 combination, 8 steps: its 1320 grids in shared memory (the largest of
+// 4096 nodes; the rest of the time is shared-memory and FP64 latency with eight
+// warps per SM) 13.35 -> 12.5 ms, its five grids in global memory 9.4 -> 5.8.
 #pragma once
 #include <cooperative_groups.h>
 

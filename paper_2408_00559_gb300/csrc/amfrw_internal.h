@@ -325,16 +325,17 @@ constexpr int kLeanScratch = 4;  // FP64 global-memory groups: the smallest slic
 
 // FP64 grids on whole blocks (amfrw_f64.cuh): offsets of a grid's arrays.  CTA
 // groups keep the vectors the stencil reads (Z, K1, Kw) and the small tables in
-// shared memory, then what fits of the central differences (single blocks),
-// the right-hand sides K0 (clusters: their barriers empty the L1 cache), the
-// line-solve factors and the tables by rate index, the rest in the slice of
-// global scratch; global-memory groups keep everything there.
+// shared memory, then what fits the class's budget of the central differences
+// (single blocks), the right-hand sides K0 (clusters: their barriers empty the
+// L1 cache), the line-solve factors and the tables by rate index, the rest in
+// the slice of global scratch; global-memory groups keep everything there.
 constexpr int kF64SmemMax = 224 * 1024;
 constexpr int kMaxCluster = 8;
 
 // log2 of the lanes among which the lines of a solve are spread: all warps of
 // a block; half of a cluster's, whose lines are short enough by then (65x65
-// grid on eight blocks: 1.25 ms with a quarter, 1.04 with half).
+// grid on eight blocks: 1.25 ms with a quarter, 1.04 with half, each before
+// factors were loaded ahead).
 AMFRW_HD int f64_tlog(int csize, int block)
 {
     int c = 0, b = 0;
