@@ -60,11 +60,13 @@ struct Slab {
 // cycles away and a store waits for it, so the rows of a batch are loaded
 // first, computed side by side, and stored last; elimination, the one chain,
 // takes a single multiply-add per row each way.  MANY: there are several
-// batches, and a batch's rows and factors are loaded while the one before it
-// is computed (a line of 16384 rows in global scratch waited for its factors at
-// every batch: 4.8 ms a step, 2.8 so; one of 4096 in shared memory, whose
-// factors do not fit there, 0.79, 0.64).  Otherwise B = R.
-template <int N, int B, bool MANY, class Get, class Put>
+// batches, and a batch's rows are loaded while the one before it is computed;
+// otherwise B = R.  AHEAD: so are its factors, which pays where they lie in
+// global scratch (a line of 16384 rows waited for them at every batch: 4.8 ms a
+// step, 2.8 so; one of 4096 rows in shared memory, whose factors do not fit
+// there, 0.79, 0.64) and not where they lie in shared memory (a d=3 level-9
+// combination, 16 steps: 1.13 ms without, 1.19 with).
+template <int N, int B, bool MANY, bool AHEAD, class Get, class Put>
 __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, const double* lu, double* dst, const Slab& sl,
                                                int cls0, int tid, int nt, Get get, Put put)
 {
@@ -109,8 +111,10 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
             double prev = 0.0;  // the row before the batch, as it was
             double al[B], ga[B];
             rows(x, act, 0);
-            factors(al, act, 0, 2 * k);
-            factors(ga, act, 0, 2 * k + 1);
+            if constexpr (AHEAD || !MANY) {
+                factors(al, act, 0, 2 * k);
+                factors(ga, act, 0, 2 * k + 1);
+            }
 #pragma unroll 1
             for (int q0 = 0; q0 < R; q0 += B) {
                 double nx[B], na[B], ng[B], v[B];
@@ -118,13 +122,20 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
                 if constexpr (MANY) {
                     const bool more = act && q0 + B < R;
                     rows(nx, more, q0 + B);
-                    factors(na, more, q0 + B, 2 * k);
-                    factors(ng, more, q0 + B, 2 * k + 1);
+                    if constexpr (AHEAD) {
+                        factors(na, more, q0 + B, 2 * k);
+                        factors(ng, more, q0 + B, 2 * k + 1);
+                    }
                 }
 #pragma unroll
                 for (int i = 0; i < B; ++i) {
                     const double vm = shfl(send_prev ? (i > 0 ? x[i > 0 ? i - 1 : 0] : prev) : x[i], sm, P, 0xffffffffu);
                     const double vp = shfl(send_next ? (i < B - 1 ? x[i < B - 1 ? i + 1 : i] : nx[0]) : x[i], sp, P, 0xffffffffu);
+                    if constexpr (MANY && !AHEAD) {
+                        const double* row = tb + (q0 + i) * PS + 2 * k;
+                        al[i] = act ? row[0] : 0.0;
+                        ga[i] = act ? row[1] : 0.0;
+                    }
                     v[i] = fma(-ga[i], vp, fma(-al[i], vm, x[i]));
                 }
                 prev = x[B - 1];
@@ -136,8 +147,10 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
 #pragma unroll
                     for (int i = 0; i < B; ++i) {
                         x[i] = nx[i];
-                        al[i] = na[i];
-                        ga[i] = ng[i];
+                        if constexpr (AHEAD) {
+                            al[i] = na[i];
+                            ga[i] = ng[i];
+                        }
                     }
                 }
             }
@@ -147,21 +160,28 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
             const int e = 2 * plog;
             double y = 0.0, lo[B], iv[B];
             rows(x, true, 0);
-            factors(lo, true, 0, e);
-            factors(iv, true, 0, e + 1);
+            if constexpr (AHEAD || !MANY) {
+                factors(lo, true, 0, e);
+                factors(iv, true, 0, e + 1);
+            }
 #pragma unroll 1
             for (int q0 = 0; q0 < R; q0 += B) {
                 double nx[B], nlo[B], niv[B];
                 const bool more = MANY && q0 + B < R;
                 if constexpr (MANY) {
                     rows(nx, more, q0 + B);
-                    factors(nlo, more, q0 + B, e);
-                    factors(niv, more, q0 + B, e + 1);
+                    if constexpr (AHEAD) {
+                        factors(nlo, more, q0 + B, e);
+                        factors(niv, more, q0 + B, e + 1);
+                    } else {
+                        factors(iv, true, q0, e + 1);
+                    }
                 }
 #pragma unroll
                 for (int i = 0; i < B; ++i) x[i] *= iv[i];
 #pragma unroll
                 for (int i = 0; i < B; ++i) {
+                    if constexpr (MANY && !AHEAD) lo[i] = tb[(q0 + i) * PS + e];
                     if (i > 0 || q0 > 0) x[i] = fma(-lo[i], y, x[i]);
                     y = x[i];
                 }
@@ -172,25 +192,28 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
 #pragma unroll
                         for (int i = 0; i < B; ++i) {
                             x[i] = nx[i];
-                            lo[i] = nlo[i];
-                            iv[i] = niv[i];
+                            if constexpr (AHEAD) {
+                                lo[i] = nlo[i];
+                                iv[i] = niv[i];
+                            }
                         }
                     }
                 }
             }
             // back from the last batch, which is still in x
             double up[B];
-            factors(up, true, R - B, e + 2);
+            if constexpr (AHEAD || !MANY) factors(up, true, R - B, e + 2);
             first = false;
 #pragma unroll 1
             for (int q0 = R - B; q0 >= 0; q0 -= B) {
                 double nx[B], nup[B];
                 if constexpr (MANY) {
                     rows(nx, q0 > 0, q0 - B);
-                    factors(nup, q0 > 0, q0 - B, e + 2);
+                    if constexpr (AHEAD) factors(nup, q0 > 0, q0 - B, e + 2);
                 }
 #pragma unroll
                 for (int i = B - 1; i >= 0; --i) {
+                    if constexpr (MANY && !AHEAD) up[i] = tb[(q0 + i) * PS + e + 2];
                     if (i < B - 1 || q0 + B < R) x[i] = fma(-up[i], y, x[i]);
                     y = x[i];
                 }
@@ -200,7 +223,7 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
 #pragma unroll
                     for (int i = 0; i < B; ++i) {
                         x[i] = nx[i];
-                        up[i] = nup[i];
+                        if constexpr (AHEAD) up[i] = nup[i];
                     }
                 }
             }
@@ -208,15 +231,18 @@ __device__ __forceinline__ void sweep_f64_rows(const Shape<N>& s, int axis, cons
     }
 }
 
+// fast: the factors lie in shared memory (or, from five axes on, where long lines
+// are rare in grids that fit there, may as well).
 template <int N, class Get, class Put>
-__device__ __forceinline__ void sweep_f64(const Shape<N>& s, int axis, const double* lu, double* dst, const Slab& sl,
-                                          int cls0, int tid, int nt, Get get, Put put)
+__device__ __forceinline__ void sweep_f64(const Shape<N>& s, int axis, const double* lu, bool fast, double* dst,
+                                          const Slab& sl, int cls0, int tid, int nt, Get get, Put put)
 {
     const int R = s.M[axis] >> s.plog[axis];
-    if (R > 4) sweep_f64_rows<N, 4, true>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
-    else if (R == 4) sweep_f64_rows<N, 4, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
-    else if (R == 2) sweep_f64_rows<N, 2, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
-    else sweep_f64_rows<N, 1, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    if (R > 4 && !fast) sweep_f64_rows<N, 4, true, true>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else if (R > 4) sweep_f64_rows<N, 4, true, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else if (R == 4) sweep_f64_rows<N, 4, false, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else if (R == 2) sweep_f64_rows<N, 2, false, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
+    else sweep_f64_rows<N, 1, false, false>(s, axis, lu, dst, sl, cls0, tid, nt, get, put);
 }
 
 template <int N, int KIND>
@@ -509,7 +535,7 @@ __device__ void solve_item_f64(const SolveArgs& a, const Item& it, unsigned char
             if ((s.skip >> ax) & 1) continue;
             const bool far = remote && ax == sl.x && (src != K0 || k0_fast);
             sweep_f64<N>(
-                s, ax, lu + lu_at(ax), to, sl, ax == 0 && own0 ? crank * (s.M[N - 1] >> sl.c) : 0, tid, nt,
+                s, ax, lu + lu_at(ax), !MEM && (lu_fast || N > 4), to, sl, ax == 0 && own0 ? crank * (s.M[N - 1] >> sl.c) : 0, tid, nt,
                 [&](int t, int J) -> double {
                     return far ? *cg::cluster_group::map_shared_rank(const_cast<double*>(src) + J, sl.owner(t)) : src[J];
                 },
