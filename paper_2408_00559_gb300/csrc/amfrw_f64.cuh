@@ -27,7 +27,7 @@
 // shared memory.
 // A class with more grids than SMs runs one, two or four blocks per SM, each
 // with its part of the shared memory (f64_widths in amfrw_api.cu).
-// Measured, before this kernel -> now: 65x65 full grid, 20 steps, 4.31 -> 0.94
+// Measured, before this kernel -> now: 65x65 full grid, 20 steps, 4.31 -> 0.95
 // ms (eight blocks); 120 grids of 128 nodes, 10 steps, 0.46 -> 0.24 ms; a d=4
 // level-12 combination, 8 steps: its 1320 grids in shared memory (the largest of
 // 4096 nodes; the rest of the time is shared-memory and FP64 latency with eight
